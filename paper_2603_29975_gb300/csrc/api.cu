@@ -46,20 +46,23 @@ static EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// 3-D fp16 map over [planes][rows][kdim] (row pitch kpad elements), box {16, box_rows, box_planes}
-static ozk_status_t make_slice_map(CUtensorMap* map, void* base, long long kdim, long long kpad, long long rows,
-                                   long long planes, int box_rows, int box_planes) {
+// Map over the digit planes [batch][halves][S][rows][8 fp16] in 8-byte elements (a row of a half is
+// two of them), box: two halves of S slices of box_rows rows; positions past the plane read zero.
+static ozk_status_t make_slice_map(CUtensorMap* map, void* base, long long halves, long long rows, long long batch,
+                                   int S, int box_rows) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return set_error(OZK_ERR_CUDA, "cuTensorMapEncodeTiled entry point unavailable");
-  cuuint64_t dims[3] = {static_cast<cuuint64_t>(kdim), static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(planes)};
-  cuuint64_t strides[2] = {static_cast<cuuint64_t>(kpad) * 2, static_cast<cuuint64_t>(rows) * kpad * 2};
-  cuuint32_t box[3] = {16u, static_cast<cuuint32_t>(box_rows), static_cast<cuuint32_t>(box_planes)};
-  cuuint32_t es[3] = {1u, 1u, 1u};
-  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  const cuuint64_t run = static_cast<cuuint64_t>(rows) * 16, half = run * static_cast<cuuint64_t>(S);
+  cuuint64_t dims[4] = {static_cast<cuuint64_t>(rows) * 2, static_cast<cuuint64_t>(S), static_cast<cuuint64_t>(halves),
+                        static_cast<cuuint64_t>(batch)};
+  cuuint64_t strides[3] = {run, half, half * static_cast<cuuint64_t>(halves)};
+  cuuint32_t box[4] = {static_cast<cuuint32_t>(2 * box_rows), static_cast<cuuint32_t>(S), 2u, 1u};
+  cuuint32_t es[4] = {1u, 1u, 1u, 1u};
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     char m[160];
-    std::snprintf(m, sizeof(m), "cuTensorMapEncodeTiled failed (%d) dims %lld %lld %lld", static_cast<int>(r), kdim, rows, planes);
+    std::snprintf(m, sizeof(m), "cuTensorMapEncodeTiled failed (%d) dims %lld %d %lld %lld", static_cast<int>(r), rows, S, halves, batch);
     return set_error(OZK_ERR_CUDA, m);
   }
   return OZK_OK;
@@ -295,7 +298,7 @@ ozk_status_t plan_gemm(const EmuGemm& g, GemmPlan* P) {
   P->rowsA = std::max(g.mmax, 1);
   P->rowsB = 2 * std::max(g.nmax, 1);
   const size_t stage = static_cast<size_t>(S) * (128 + P->BN) * 32;
-  P->nstage = static_cast<int>(std::min<size_t>(6, (200 * 1024 - 2048) / stage));
+  P->nstage = static_cast<int>(std::min<size_t>(6, (227 * 1024 - 14 * 1024) / stage));
   if (P->nstage < 1) return set_error(OZK_ERR_ARG, "S too large for the shared-memory pipeline");
   P->kblocks = static_cast<int>((kp2 + 15) / 16);
   // exactness chunk: every product of two digits is <= 2^14 in magnitude; an FP32 accumulator
@@ -367,8 +370,6 @@ ozk_status_t run_emulated(ozk_context* h, const EmuGemm& g, size_t ws_offset = 0
   sp.trans = g.oa.trans; sp.conj = g.oa.conj; sp.side = 0;
   sp.out_rows = P.rowsA; sp.out = As; sp.exps = e; sp.exp_stride = P.rowsA;
   sp.dbg_digits = g.dbg_digits_a;
-  sp.gmax = reinterpret_cast<unsigned long long*>(ws + P.offGA);
-  sp.kgroups = 1;
   if (single) { sp.X = nullptr; sp.X1 = g.A; sp.ld1 = g.lda; sp.rows1 = g.m; sp.k1 = g.k; sp.zstride1 = g.zsA; }
   else { sp.X = g.tA; sp.ld = g.tlda; sp.rows = g.tm; sp.kdim = g.tk; }
   const double smnk = g.sum_mnk >= 0 ? g.sum_mnk : static_cast<double>(g.m) * g.n * g.k;
@@ -379,7 +380,6 @@ ozk_status_t run_emulated(ozk_context* h, const EmuGemm& g, size_t ws_offset = 0
   sq.trans = g.ob.trans ? 0 : 1; sq.conj = g.ob.conj; sq.side = 1;
   sq.out_rows = P.rowsB; sq.out = Bs; sq.exps = f; sq.exp_stride = std::max(g.nmax, 1);
   sq.dbg_digits = nullptr;
-  sq.gmax = reinterpret_cast<unsigned long long*>(ws + P.offGB);
   if (single) { sq.X = nullptr; sq.X1 = g.B; sq.ld1 = g.ldb; sq.rows1 = g.n; sq.k1 = g.k; sq.zstride1 = g.zsB; }
   else { sq.X = g.tB; sq.ld = g.tldb; sq.rows = g.tn; sq.kdim = g.tk; }
   const bool split_a = (g.split_sides & 1) != 0, split_b = (g.split_sides & 2) != 0;
@@ -403,9 +403,9 @@ ozk_status_t run_emulated(ozk_context* h, const EmuGemm& g, size_t ws_offset = 0
   if (!g.run_gemm) return cuda_check(cudaGetLastError(), "split launch");
 
   CUtensorMap ta, tb;
-  st = make_slice_map(&ta, As, 2LL * g.kmax, P.kpad, P.rowsA, static_cast<long long>(S) * g.batch, 128, S);
+  st = make_slice_map(&ta, As, P.kpad / 8, P.rowsA, g.batch, S, 128);
   if (st) return st;
-  st = make_slice_map(&tb, Bs, 2LL * g.kmax, P.kpad, P.rowsB, static_cast<long long>(S) * g.batch, P.BN, S);
+  st = make_slice_map(&tb, Bs, P.kpad / 8, P.rowsB, g.batch, S, P.BN);
   if (st) return st;
 
   GemmParams gp{};
@@ -441,6 +441,7 @@ ozk_status_t run_emulated(ozk_context* h, const EmuGemm& g, size_t ws_offset = 0
   h->stall_next = 0;
   gp.resid = g.resid; gp.ldres = g.ldres;
   gp.ar = g.ar; gp.ai = g.ai; gp.br = g.br; gp.bi = g.bi;
+  gp.unit_alpha = (g.ar == 1.0 && g.ai == 0.0) ? 1 : 0;
   if (g.mode >= 0) gp.mode = g.mode;
   else if (g.br == 0.0 && g.bi == 0.0) gp.mode = 0;
   else if (g.ar == -1.0 && g.ai == 0.0 && g.br == 1.0 && g.bi == 0.0) gp.mode = 1;
@@ -448,7 +449,7 @@ ozk_status_t run_emulated(ozk_context* h, const EmuGemm& g, size_t ws_offset = 0
   gp.e = e; gp.f = f; gp.e_stride = P.rowsA; gp.f_stride = std::max(g.nmax, 1);
   gp.groups = g.groups; gp.status = h->d_status;
   if (single) { gp.m = nullptr; gp.m1 = g.m; gp.n1 = g.n; gp.C1 = g.C; gp.ldc1 = g.ldc; gp.skm1 = g.skm; gp.skn1 = g.skn; }
-  else { gp.m = g.tm; gp.n = g.tn; gp.C = g.tC; gp.ldc = g.tldc; gp.skm = g.tskm; gp.skn = g.tskn; }
+  else { gp.m = g.tm; gp.n = g.tn; gp.k = g.tk; gp.C = g.tC; gp.ldc = g.tldc; gp.skm = g.tskm; gp.skn = g.tskn; }
   gp.crow = g.crow; gp.crow_b = g.crow_b; gp.crow_n = g.crow_n; gp.crow_perm = g.crow_perm;
   if (g.remap) {
     gp.remap = reinterpret_cast<const int2*>(g.remap);

@@ -70,8 +70,15 @@ __global__ void __launch_bounds__(RS_THREADS) residue_split_kernel(const SplitPa
   }
   __syncthreads();
   const int N = T.N;
-  const long long plane = p.out_rows * p.kpad;
-  __half* outz = p.out + static_cast<long long>(z) * N * plane;
+  // planes in the layout of the slice split (one plane per modulus)
+  const int halves = static_cast<int>(p.kpad >> 3);
+  __half* outz = p.out + static_cast<long long>(z) * halves * N * p.out_rows * 8;
+  auto at = [&](int t, long long row, int l, int second) -> __half& {
+    const int kb = l >> 3, q = l & 7;
+    const bool tail4 = K - 8 * kb <= 4;                 // packed into the first half
+    const int half = 2 * kb + (tail4 ? 0 : second), pos = tail4 ? 4 * second + q : q;
+    return outz[((static_cast<long long>(half) * N + t) * p.out_rows + row) * 8 + pos];
+  };
   const int nr = min(RS_ROWS, R - r0);
   // stored row-fastest (trans == 0: rows of 32 consecutive threads) or column-fastest
   const int span = p.trans ? nr * K : RS_ROWS * K;
@@ -99,30 +106,34 @@ __global__ void __launch_bounds__(RS_THREADS) residue_split_kernel(const SplitPa
 #pragma unroll
       for (int s = 0; s < 8; ++s) { ar += dr[s] * T.pow256[t][s]; ai += di[s] * T.pow256[t][s]; }
       const int rr = sym_mod(ar, T.mod[t]), ri = sym_mod(ai, T.mod[t]);
-      __half* o = outz + t * plane;
       if (p.side == 0) {
-        o[r * p.kpad + l] = __int2half_rn(rr);
-        o[r * p.kpad + K + l] = __int2half_rn(ri);
+        at(t, r, l, 0) = __int2half_rn(rr);
+        at(t, r, l, 1) = __int2half_rn(ri);
       } else {
         const long long row0 = 2LL * r, row1 = 2LL * r + 1;
-        o[row0 * p.kpad + l] = __int2half_rn(rr);
-        o[row0 * p.kpad + K + l] = __int2half_rn(-ri);
-        o[row1 * p.kpad + l] = __int2half_rn(ri);
-        o[row1 * p.kpad + K + l] = __int2half_rn(rr);
+        at(t, row0, l, 0) = __int2half_rn(rr);
+        at(t, row0, l, 1) = __int2half_rn(-ri);
+        at(t, row1, l, 0) = __int2half_rn(ri);
+        at(t, row1, l, 1) = __int2half_rn(rr);
       }
     }
   }
-  // zero the K padding [2K, kpad) of the rows this CTA owns
-  const int pad = static_cast<int>(p.kpad) - 2 * K;
-  if (pad > 0) {
+  // zero the positions of the last K-block past K (of the rows this CTA owns)
+  const int rem = K & 7;
+  if (rem) {
+    const int kb = K >> 3, width = rem <= 4 ? 4 : 8;   // positions per scalar in use
     const int rows_out = p.side == 0 ? 1 : 2;
-    const int nro = nr * rows_out;
-    for (int idx = tid; idx < N * nro * pad; idx += RS_THREADS) {
-      const int c = idx % pad;
-      const int rr = (idx / pad) % nro;
-      const int t = idx / (pad * nro);
-      outz[t * plane + (static_cast<long long>(r0) * rows_out + rr) * p.kpad + 2 * K + c] = __float2half(0.0f);
+    const int nro = nr * rows_out, gap = width - rem;
+    for (int idx = tid; idx < N * nro * gap * 2; idx += RS_THREADS) {
+      const int second = idx & 1, q = (idx >> 1) % gap, rr = (idx >> 1) / gap % nro, t = (idx >> 1) / (gap * nro);
+      at(t, static_cast<long long>(r0) * rows_out + rr, 8 * kb + rem + q, second) = __float2half(0.0f);
     }
+    if (rem <= 4 && 2 * kb + 1 < halves)
+      for (int idx = tid; idx < N * nro * 8; idx += RS_THREADS) {
+        const int q = idx & 7, rr = (idx >> 3) % nro, t = (idx >> 3) / nro;
+        outz[((static_cast<long long>(2 * kb + 1) * N + t) * p.out_rows + static_cast<long long>(r0) * rows_out + rr) * 8 +
+             q] = __float2half(0.0f);
+      }
   }
 }
 

@@ -131,11 +131,14 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t by
                ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
 
+// Waits up to about a millisecond (the suspend-time hint, in ns) before it answers: with the default
+// limit the waiting threads of a tensor-core CTA came back every few tens of cycles and their polling
+// took about a third of the issue slots of every SM sub-partition.
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
-      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity), "r"(1000000u) : "memory");
   return ok != 0;
 }
 
@@ -143,9 +146,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // sets OZK_ERR_TIMEOUT in *status and the CTA-local abort flag, and returns false.
 constexpr long long kWaitBudget = 2000000000LL;
 
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* status,
-                                          volatile int* abort_flag, long long budget = kWaitBudget) {
-  if (mbar_try_wait(bar, parity)) return true;
+__device__ __forceinline__ bool mbar_wait_more(uint64_t* bar, uint32_t parity, int* status, volatile int* abort_flag,
+                                                   long long budget) {
   const long long t0 = clock64();
   while (true) {
     if (mbar_try_wait(bar, parity)) return true;
@@ -157,15 +159,26 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* s
     }
   }
 }
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* status,
+                                          volatile int* abort_flag, long long budget = kWaitBudget) {
+  return mbar_try_wait(bar, parity) || mbar_wait_more(bar, parity, status, abort_flag, budget);
+}
+
+// One thread of a converged warp, the same one at every call.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+  return p != 0;
+}
 
 // ------------------------------------------------------------------ TMA
-__device__ __forceinline__ void tma_load_3d(const CUtensorMap* map, void* smem_dst, uint64_t* bar,
-                                            int c0, int c1, int c2) {
+__device__ __forceinline__ void tma_load_4d(const CUtensorMap* map, void* smem_dst, uint64_t* bar,
+                                            int c0, int c1, int c2, int c3) {
   asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4, %5}], [%2];"
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%3, %4, %5, %6}], [%2];"
       ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)),
-        "r"(c0), "r"(c1), "r"(c2)
+        "r"(c0), "r"(c1), "r"(c2), "r"(c3)
       : "memory");
 }
 
@@ -191,15 +204,15 @@ __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// K-major operand tile in shared memory with the 32-byte swizzle: rows of 32 bytes
-// (16 fp16 = one MMA K step), 8-row groups 256 bytes apart.
-__device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t saddr) {
+// K-major operand tile in shared memory without swizzle: core matrices of 8 rows x 16 bytes, the
+// rows of one 16-byte K half back to back (8-row groups 128 bytes apart) and the second half of an
+// MMA's K step (16 fp16) `half_bytes` after the first.
+__device__ __forceinline__ uint64_t smem_desc_halves(uint32_t saddr, uint32_t half_bytes) {
   uint64_t d = 0;
   d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
-  d |= static_cast<uint64_t>(1) << 16;                 // leading byte offset (unused here)
-  d |= static_cast<uint64_t>(256u >> 4) << 32;         // stride byte offset: 8 rows x 32 B
+  d |= static_cast<uint64_t>(half_bytes >> 4) << 16;   // leading byte offset: K direction
+  d |= static_cast<uint64_t>(128u >> 4) << 32;         // stride byte offset: rows
   d |= static_cast<uint64_t>(1) << 46;                 // descriptor version
-  d |= static_cast<uint64_t>(6) << 61;                 // swizzle: 32 B
   return d;
 }
 

@@ -17,8 +17,8 @@ struct SplitParams {
   int S;
   int nbits;                // B = 8S - 1
   long long out_rows;       // row count of one slice plane
-  long long kpad;           // row pitch (fp16 elements)
-  __half* out;              // [batch][S][out_rows][kpad]
+  long long kpad;           // fp16 elements kept per row (2 K rounded up to 8): kpad / 8 halves
+  __half* out;              // [batch][kpad / 8][S][out_rows][8] (layout: split.cu)
   int* exps;                // [batch][exp_stride]
   long long exp_stride;
   int16_t* dbg_digits;      // optional int16 copy [S][out_rows][2k] for problem 0 (test hook)
@@ -27,12 +27,7 @@ struct SplitParams {
   // uniform batch starts at X1 + z * zstride1
   const double2* X1; int ld1, rows1, k1;
   long long zstride1;
-  // K-parallel split (operands with few row blocks and long rows): gmax[z exp_stride + r] holds
-  // the bit pattern of row r's largest |Re|, |Im| (taken by split_rowmax_kernel over K
-  // segments), and kgroups CTAs share each row block's K tiles; kgroups <= 1: one CTA per row
-  // block scans and splits the whole row
-  unsigned long long* gmax;
-  int kgroups;
+  int kgroups;              // CTAs (a cluster) that share a row block's K-blocks (set by the launcher)
 };
 struct SplitPair { SplitParams s[2]; int nsides; };
 
@@ -73,7 +68,7 @@ struct GemmParams {
   int S;
   int npairs;
   int ngroups;            // G = g_max - 1
-  int kblocks;            // K' / 16 rounded up (uniform over the batch)
+  int kblocks;            // K-blocks of 16 digits (8 complex elements), the largest over the batch
   int chunk_kb;           // K-blocks per exactness chunk
   int nstage;
   int mode;
@@ -90,10 +85,12 @@ struct GemmParams {
   // tiles enumerated per problem (set by the launcher): only tiles not wholly inside a box
   int box_m, box_n, tpp;
   double ar, ai, br, bi;  // alpha, beta
+  int unit_alpha;         // alpha == 1 (a test that keeps the epilogue off the FP64 pipe)
   const int* m;           // per problem rows of C
   const int* n;           // per problem complex columns of C
   double2* const* C;      // per problem output pointer
   const int* ldc;
+  const int* k;           // per problem K (null: kblocks K-blocks in every problem)
   const int* e;           // exponents of rows  [batch][e_stride]
   const int* f;           // exponents of cols  [batch][f_stride]
   long long e_stride, f_stride;

@@ -1,13 +1,20 @@
 // Exponent scan and slice split (paper Sec. 2.2: slices by significant bits with exponent
-// alignment).  One CTA owns 32 logical rows of an operand: it reads them once to find the
-// per-row maximum of |Re| and |Im| (integer compare on the binary64 bit patterns), derives
-// the frexp exponent, then reads them again (from L2) and writes the S balanced int8 digits
-// of every real scalar as fp16 values in the K-major stacked layout the tensor-core kernel
-// loads with TMA:
-//   left operand  (side 0): out[z][s][r][l]     = digit of Re x_rl, out[z][s][r][k+l] = Im
-//   right operand (side 1): out[z][s][2r][l]    = Re,  out[z][s][2r][k+l]   = -Im (digit-wise)
-//                           out[z][s][2r+1][l]  = Im,  out[z][s][2r+1][k+l] = Re
-// Positions [2k, kpad) of every written row are zero.  All integer work, no FP64 arithmetic.
+// alignment).  The S balanced int8 digits of every real scalar of an operand are written as fp16
+// values in the K-major layout the tensor-core kernel loads with TMA:
+//   out[z][h][s][row][8]   (8 fp16 = 16 bytes: one row of a tensor-core core matrix)
+// K-block kb covers the elements l = 8 kb .. 8 kb + 7 of a row; half h = 2 kb holds the digits of
+// their first scalar, h = 2 kb + 1 those of the second:
+//   left operand  (side 0): row r       first Re x_rl, second Im x_rl
+//   right operand (side 1): row 2r      first Re,      second -Im (digit-wise)
+//                           row 2r + 1  first Im,      second Re
+// (sums over K run over all the halves, so their order is free).  A last K-block of at most 4
+// elements is packed into half 2 kb alone: 4 values of the first scalar, then 4 of the second;
+// the half after it is zero where the plane has one.  Rows follow each other at 16 bytes for a
+// fixed (h, s), so the 32 lanes of a warp, one row each, store 512 (left) or 1024 (right)
+// contiguous bytes, and a 128-row operand tile is 2 S runs of 2 KB for the TMA (with the digits of
+// a row K-contiguous instead, the tile's runs are the 32 bytes of a K-block and row: 1344 of them
+// for S = 7, which the TMA fetches at about one per clock, 656 ns per K-block measured with the
+// tensor work left out).  All integer work, no FP64 arithmetic.
 #include <algorithm>
 #include <type_traits>
 
@@ -15,84 +22,12 @@
 
 namespace ozk {
 
+constexpr int SPLIT_ROWS = 32;               // rows of a CTA: one per lane
+constexpr int SPLIT_MAX_WARPS = 8;           // a warp takes one K-block (8 elements) at a time
+constexpr int SPLIT_MAX_KG = 8;              // CTAs of a cluster that share a row block's K-blocks
 
-
-constexpr int SPLIT_ROWS = 32;
-constexpr int SPLIT_TK = 64;
-constexpr int SPLIT_THREADS = 256;
-
-// PER consecutive fp16 values (digits d[0..PER-1], negated when NEG) stored as one aligned
-// vector at dst.
-template <int PER, bool NEG>
-__device__ __forceinline__ void store_digits(__half* dst, const int (&d)[PER]) {
-  __half h[PER];
-#pragma unroll
-  for (int q = 0; q < PER; ++q) h[q] = __int2half_rn(NEG ? -d[q] : d[q]);
-  if constexpr (PER == 8) {
-    uint4 v;
-    v.x = __half_as_ushort(h[0]) | (static_cast<uint32_t>(__half_as_ushort(h[1])) << 16);
-    v.y = __half_as_ushort(h[2]) | (static_cast<uint32_t>(__half_as_ushort(h[3])) << 16);
-    v.z = __half_as_ushort(h[4]) | (static_cast<uint32_t>(__half_as_ushort(h[5])) << 16);
-    v.w = __half_as_ushort(h[6]) | (static_cast<uint32_t>(__half_as_ushort(h[7])) << 16);
-    *reinterpret_cast<uint4*>(dst) = v;
-  } else if constexpr (PER == 4) {
-    uint2 v;
-    v.x = __half_as_ushort(h[0]) | (static_cast<uint32_t>(__half_as_ushort(h[1])) << 16);
-    v.y = __half_as_ushort(h[2]) | (static_cast<uint32_t>(__half_as_ushort(h[3])) << 16);
-    *reinterpret_cast<uint2*>(dst) = v;
-  } else if constexpr (PER == 2) {
-    *reinterpret_cast<uint32_t*>(dst) = __half_as_ushort(h[0]) | (static_cast<uint32_t>(__half_as_ushort(h[1])) << 16);
-  } else {
-    *dst = h[0];
-  }
-}
-
-// Digits of PER consecutive elements of one row (positions l .. l + PER - 1, all < K, l and K
-// multiples of PER), every slice written with vector stores.  W64: 64-bit integer images
-// (nbits <= 62), else 128-bit.
-template <int PER, bool W64>
-__device__ __forceinline__ void split_run(const SplitParams& p, const double2* v, int e, int r, int l, int K,
-                                          __half* outz, long long plane) {
-  using Int = typename std::conditional<W64, long long, __int128>::type;
-  Int Xr[PER], Xi[PER];
-#pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    if constexpr (W64) {
-      Xr[q] = integer_image64(v[q].x, e, p.nbits);
-      Xi[q] = integer_image64(v[q].y, e, p.nbits);
-    } else {
-      Xr[q] = integer_image(v[q].x, e, p.nbits);
-      Xi[q] = integer_image(v[q].y, e, p.nbits);
-    }
-  }
-  for (int s = p.S - 1; s >= 0; --s) {
-    int dr[PER], di[PER];
-#pragma unroll
-    for (int q = 0; q < PER; ++q) {
-      if constexpr (W64) {
-        dr[q] = s ? next_digit64(Xr[q]) : static_cast<int>(Xr[q]);
-        di[q] = s ? next_digit64(Xi[q]) : static_cast<int>(Xi[q]);
-      } else {
-        dr[q] = s ? next_digit(Xr[q]) : static_cast<int>(Xr[q]);
-        di[q] = s ? next_digit(Xi[q]) : static_cast<int>(Xi[q]);
-      }
-    }
-    __half* o = outz + s * plane;
-    if (p.side == 0) {
-      store_digits<PER, false>(o + r * p.kpad + l, dr);
-      store_digits<PER, false>(o + r * p.kpad + K + l, di);
-    } else {
-      const long long row0 = 2LL * r, row1 = 2LL * r + 1;
-      store_digits<PER, false>(o + row0 * p.kpad + l, dr);
-      store_digits<PER, true>(o + row0 * p.kpad + K + l, di);
-      store_digits<PER, false>(o + row1 * p.kpad + l, di);
-      store_digits<PER, false>(o + row1 * p.kpad + K + l, dr);
-    }
-  }
-}
-
-// The same digits for a compile-time slice count SF (nbits = 8 SF - 1, 64-bit images), with
-// no dependent chain per digit.  With C = 128 (1 + 256 + ... + 256^(SF-2)), Y = X + C holds
+// Digits of 8 elements for a compile-time slice count SF <= 8 (nbits = 8 SF - 1, 64-bit images),
+// with no dependent chain per digit.  With C = 128 (1 + 256 + ... + 256^(SF-2)), Y = X + C holds
 // the balanced digits d_s + 128 of the SF - 1 lower places as its low bytes and the top digit
 // as Y >> 8 (SF - 1): X = sum_s d_s 256^s with every lower d_s in [-128, 127], so adding 128
 // at each lower place lifts it into [0, 255] without carries, and base-256 digits are unique.
@@ -100,31 +35,12 @@ __device__ __forceinline__ void split_run(const SplitParams& p, const double2* v
 // offset by 0x6580 = (bit pattern of 1536 in binary16) - 128, which makes each half the bit
 // pattern of 1536 + d (the binade [1024, 2048) has unit spacing); one packed subtraction of
 // 1536 leaves d, and subtracting the word from 1536 leaves -d, both exact (+0 for d = 0, as
-// the int -> half conversion gives).  The top digit (|d| <= 128) takes the offset 0x6600.
+// the int -> half conversion gives).  The top digit (|d| <= 128) takes the offset 0x6600; for
+// SF = 8 (|X| < 2^63, so X + C may pass 2^63) it is taken from floor((X + C) / 2), C being even.
 __host__ __device__ constexpr long long digit_bias(int S) {
   long long c = 0;
   for (int s = 0; s < S - 1; ++s) c = c * 256 + 128;
   return c;
-}
-
-struct Y64 { uint32_t lo, hi; };
-
-// biased binary16 pair (bit patterns of 1536 + d) of plane `s` for two elements
-template <int SF>
-__device__ __forceinline__ uint32_t biased_pair(int s, Y64 a, Y64 b) {
-  if (s > 0) {
-    const int k = SF - 1 - s;                               // byte of Y, 0 .. SF - 2
-    const uint32_t wa = k < 4 ? a.lo : a.hi, wb = k < 4 ? b.lo : b.hi;
-    const uint32_t kk = static_cast<uint32_t>(k & 3);
-    const uint32_t w = __byte_perm(wa, wb, kk | ((kk + 4u) << 8));
-    return (w & 0x00FF00FFu) + 0x65806580u;
-  }
-  constexpr int sh = 8 * (SF - 1);
-  const long long ya = static_cast<long long>((static_cast<unsigned long long>(a.hi) << 32) | a.lo);
-  const long long yb = static_cast<long long>((static_cast<unsigned long long>(b.hi) << 32) | b.lo);
-  const uint32_t ta = static_cast<uint32_t>(static_cast<int>(ya >> sh) + 0x6600);
-  const uint32_t tb = static_cast<uint32_t>(static_cast<int>(yb >> sh) + 0x6600);
-  return __byte_perm(ta, tb, 0x5410);
 }
 
 __device__ __forceinline__ uint32_t half2_bits(__half2 h) {
@@ -142,315 +58,288 @@ __device__ __forceinline__ uint32_t pair_digits(uint32_t biased) {
   return half2_bits(NEG ? __hsub2(k1536, bits_half2(biased)) : __hsub2(bits_half2(biased), k1536));
 }
 
-template <int NW>
-__device__ __forceinline__ void store_words(__half* dst, const uint32_t (&w)[NW]) {
-  if constexpr (NW == 4) *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-  else if constexpr (NW == 2) *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
-  else *reinterpret_cast<uint32_t*>(dst) = w[0];
+// the biased pair of the top digits (SF < 8) of two images Y, given by their words
+template <int SF>
+__device__ __forceinline__ uint32_t top_pair(uint32_t al, uint32_t ah, uint32_t bl, uint32_t bh) {
+  constexpr int sh = 8 * (SF - 1);
+  uint32_t ta, tb;
+  if constexpr (sh >= 32) {
+    ta = static_cast<uint32_t>((static_cast<int>(ah) >> (sh - 32)) + 0x6600);
+    tb = static_cast<uint32_t>((static_cast<int>(bh) >> (sh - 32)) + 0x6600);
+  } else {                                       // the top digit fits in 9 bits: low word after the shift
+    ta = __funnelshift_r(al, ah, sh) + 0x6600u;
+    tb = __funnelshift_r(bl, bh, sh) + 0x6600u;
+  }
+  return __byte_perm(ta, tb, 0x5410);
 }
 
-template <int PER, int SF>
-__device__ __forceinline__ void split_run_fixed(const SplitParams& p, const double2* v, int e, int r, int l, int K,
-                                                __half* outz, long long plane) {
-  static_assert(PER >= 2 && PER % 2 == 0, "pairs of elements");
+// where the digits of one row and K-block go: uint4 words of the planes (see the layout above)
+template <int SIDE>
+struct SplitDst {
+  uint4* out;                // plane (h = 2 kb, s = 0), row r (left) or 2 r (right)
+  int splane;                // uint4 words from slice s to s + 1 (= out_rows)
+  long long hplane;          // from half h to h + 1 (= S out_rows)
+  bool tail4;                // at most 4 elements: packed into the first half
+  bool has2;                 // the plane has the second half
+};
+
+// the 4 words (8 fp16) of each scalar of one slice: r first scalar, i the second, n = -i
+template <int SIDE>
+__device__ __forceinline__ void store_slice(const SplitDst<SIDE>& d, int s, const uint32_t (&r)[4], const uint32_t (&i)[4],
+                                            const uint32_t (&n)[4]) {
+  uint4* o = d.out + static_cast<long long>(s) * d.splane;
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  if (!d.tail4) {
+    if constexpr (SIDE == 0) {
+      o[0] = make_uint4(r[0], r[1], r[2], r[3]);
+      o[d.hplane] = make_uint4(i[0], i[1], i[2], i[3]);
+    } else {
+      o[0] = make_uint4(r[0], r[1], r[2], r[3]);
+      o[1] = make_uint4(i[0], i[1], i[2], i[3]);
+      o[d.hplane] = make_uint4(n[0], n[1], n[2], n[3]);
+      o[d.hplane + 1] = make_uint4(r[0], r[1], r[2], r[3]);
+    }
+  } else {
+    if constexpr (SIDE == 0) {
+      o[0] = make_uint4(r[0], r[1], i[0], i[1]);
+    } else {
+      o[0] = make_uint4(r[0], r[1], n[0], n[1]);
+      o[1] = make_uint4(i[0], i[1], r[0], r[1]);
+      if (d.has2) o[d.hplane + 1] = zero;
+    }
+    if (d.has2) o[d.hplane] = zero;
+  }
+}
+
+// The integer image X = trunc(x 2^(nbits - e)) of |x| < 2^e, nbits =
+// 8 SF - 1: the 53-bit significand, shifted left by the constant max(0, nbits - 53) that no element
+// exceeds, then right.  (Rows flagged non-finite have e = 0, which does not bound their finite
+// elements: those are cut to the significand's range.)
+template <int SF>
+__device__ __forceinline__ long long image_fixed(long long bits, int e) {
+  constexpr int nbits = 8 * SF - 1, left = nbits > 53 ? nbits - 53 : 0;
+  const int ex = static_cast<int>(bits >> 52) & 0x7FF;
+  const unsigned long long man = static_cast<unsigned long long>(bits) & ((1ull << 52) - 1ull);
+  const unsigned long long M = ex == 0 ? man : (man | (1ull << 52));
+  const int right = e + (left + 1075 - nbits) - max(ex, 1);
+  const long long mag = static_cast<long long>((M << left) >> min(max(right, 0), 63));
+  return bits < 0 ? -mag : mag;
+}
+
+template <int SF, int SIDE>
+__device__ __forceinline__ void emit_fixed(const SplitDst<SIDE>& d, const longlong2 (&v)[8], int e) {
   constexpr long long C = digit_bias(SF);
-  constexpr int NW = PER / 2;
-  Y64 yr[PER], yi[PER];
+  uint32_t rl[8], rh[8], il[8], ih[8];                    // low and high words of Y
+  uint32_t tr[4], ti[4];                                  // SF = 8: the top digits, two a word
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const unsigned long long a = static_cast<unsigned long long>(integer_image64(v[q].x, e, 8 * SF - 1) + C);
-    const unsigned long long b = static_cast<unsigned long long>(integer_image64(v[q].y, e, 8 * SF - 1) + C);
-    yr[q] = Y64{static_cast<uint32_t>(a), static_cast<uint32_t>(a >> 32)};
-    yi[q] = Y64{static_cast<uint32_t>(b), static_cast<uint32_t>(b >> 32)};
+  for (int q = 0; q < 8; ++q) {
+    const long long xr = image_fixed<SF>(v[q].x, e), xi = image_fixed<SF>(v[q].y, e);
+    const unsigned long long a = static_cast<unsigned long long>(xr) + C, b = static_cast<unsigned long long>(xi) + C;
+    rl[q] = static_cast<uint32_t>(a); rh[q] = static_cast<uint32_t>(a >> 32);
+    il[q] = static_cast<uint32_t>(b); ih[q] = static_cast<uint32_t>(b >> 32);
+    if constexpr (SF == 8) {
+      const uint32_t ta = static_cast<uint32_t>(static_cast<int>(((xr >> 1) + C / 2) >> 55) + 0x6600);
+      const uint32_t tb = static_cast<uint32_t>(static_cast<int>(((xi >> 1) + C / 2) >> 55) + 0x6600);
+      tr[q / 2] = q & 1 ? __byte_perm(tr[q / 2], ta, 0x5410) : ta;
+      ti[q / 2] = q & 1 ? __byte_perm(ti[q / 2], tb, 0x5410) : tb;
+    }
   }
 #pragma unroll
   for (int s = SF - 1; s >= 0; --s) {
-    uint32_t br[NW], bi[NW], dr[NW], di[NW];
+    const int k = SF - 1 - s;                               // byte of Y (s > 0)
+    uint32_t r[4], i[4], n[4];
 #pragma unroll
-    for (int h = 0; h < NW; ++h) {
-      br[h] = biased_pair<SF>(s, yr[2 * h], yr[2 * h + 1]);
-      bi[h] = biased_pair<SF>(s, yi[2 * h], yi[2 * h + 1]);
-      dr[h] = pair_digits<false>(br[h]);
-      di[h] = pair_digits<false>(bi[h]);
+    for (int h = 0; h < 4; ++h) {
+      uint32_t br, bi;
+      if (s > 0) {
+        const uint32_t sel = static_cast<uint32_t>(k & 3) | (static_cast<uint32_t>((k & 3) + 4) << 8);
+        br = (__byte_perm(k < 4 ? rl[2 * h] : rh[2 * h], k < 4 ? rl[2 * h + 1] : rh[2 * h + 1], sel) & 0x00FF00FFu) +
+             0x65806580u;
+        bi = (__byte_perm(k < 4 ? il[2 * h] : ih[2 * h], k < 4 ? il[2 * h + 1] : ih[2 * h + 1], sel) & 0x00FF00FFu) +
+             0x65806580u;
+      } else if constexpr (SF == 8) {
+        br = tr[h];
+        bi = ti[h];
+      } else {
+        br = top_pair<SF>(rl[2 * h], rh[2 * h], rl[2 * h + 1], rh[2 * h + 1]);
+        bi = top_pair<SF>(il[2 * h], ih[2 * h], il[2 * h + 1], ih[2 * h + 1]);
+      }
+      r[h] = pair_digits<false>(br);
+      i[h] = pair_digits<false>(bi);
+      n[h] = pair_digits<true>(bi);
     }
-    __half* o = outz + s * plane;
-    if (p.side == 0) {
-      store_words<NW>(o + static_cast<long long>(r) * p.kpad + l, dr);
-      store_words<NW>(o + static_cast<long long>(r) * p.kpad + K + l, di);
+    store_slice(d, s, r, i, n);
+  }
+}
+
+// Any S (run time): digits one at a time from 64-bit (nbits <= 62) or 128-bit images.  dbg: the
+// int16 copy of the test hook, [S][out_rows][2 K].
+template <bool W64, int SIDE>
+__device__ __forceinline__ void emit_generic(const SplitParams& p, const SplitDst<SIDE>& d, const longlong2 (&v)[8], int e,
+                                             int row, int l0, int K, int16_t* dbg) {
+  using Int = typename std::conditional<W64, long long, __int128>::type;
+  Int Xr[8], Xi[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    if constexpr (W64) {
+      Xr[q] = integer_image64(__longlong_as_double(v[q].x), e, p.nbits);
+      Xi[q] = integer_image64(__longlong_as_double(v[q].y), e, p.nbits);
     } else {
-      uint32_t ni[NW];
-#pragma unroll
-      for (int h = 0; h < NW; ++h) ni[h] = pair_digits<true>(bi[h]);
-      const long long row0 = 2LL * r, row1 = 2LL * r + 1;
-      store_words<NW>(o + row0 * p.kpad + l, dr);
-      store_words<NW>(o + row0 * p.kpad + K + l, ni);
-      store_words<NW>(o + row1 * p.kpad + l, di);
-      store_words<NW>(o + row1 * p.kpad + K + l, dr);
+      Xr[q] = integer_image(__longlong_as_double(v[q].x), e, p.nbits);
+      Xi[q] = integer_image(__longlong_as_double(v[q].y), e, p.nbits);
     }
   }
-}
-
-// Both operands of one emulated GEMM in one launch: blockIdx.z selects the side.  VEC: the
-// widest digit run stored as one vector (8 in general; 2 for K <= 16, where the runs are 2 wide
-// and the smaller register footprint keeps more CTAs resident).  W64: 64-bit integer images
-// (S <= 7).  Rows of at most SPLIT_TK elements (every panel operand of the block LU) are read
-// from global memory once: the tile is loaded, the row maxima are taken from it, then the
-// digits; longer rows take a scan pass and then the tiles one by one.
-template <int VEC, bool W64, int SF = 0>
-__global__ void __launch_bounds__(SPLIT_THREADS, VEC == 2 ? (W64 ? 5 : 4) : (W64 ? 4 : 2))
-split_kernel(const SplitPair pp) {
-  static_assert(SF == 0 || (W64 && VEC == 8), "compile-time slice counts: 64-bit images, 8-wide runs");
-  if (static_cast<int>(blockIdx.z) >= pp.nsides) return;
-  const SplitParams& p = pp.s[blockIdx.z];
-  const int z = blockIdx.y;
-  const bool single = p.X == nullptr;
-  const int R = single ? p.rows1 : p.rows[z];
-  const int K = single ? p.k1 : p.kdim[z];
-  // K-parallel: CTA x = row block x / kgroups, the kg-th share of its K tiles
-  const int kgs = p.kgroups > 1 ? p.kgroups : 1;
-  const int kg = static_cast<int>(blockIdx.x) % kgs;
-  const int r0 = (static_cast<int>(blockIdx.x) / kgs) * SPLIT_ROWS;
-  if (r0 >= R) return;
-  const double2* __restrict__ P = single ? p.X1 + z * p.zstride1 : p.X[z];
-  const long long ld = single ? p.ld1 : p.ld[z];
-  const int tid = threadIdx.x;
-  const bool kpar = kgs > 1 && K > SPLIT_TK;
-  const bool one_tile = K <= SPLIT_TK;
-
-  __shared__ unsigned long long rowmax[SPLIT_ROWS];
-  __shared__ int rowexp[SPLIT_ROWS];
-  __shared__ int rowbad[SPLIT_ROWS];
-  __shared__ double2 tile[SPLIT_ROWS][SPLIT_TK + 1];
-  __shared__ int bad;
-  if (tid < SPLIT_ROWS) { rowmax[tid] = 0ull; rowbad[tid] = 0; }
-  if (tid == 0) bad = 0;
-  __syncthreads();
-
-  // tile width along K: 64, or K rounded up to 8 for short rows (so no thread idles on padding)
-  const int TK = K >= SPLIT_TK ? SPLIT_TK : ((K + 7) & ~7);
-  const int per = TK / 8;                      // consecutive l per thread
-  // a 32 x TK tile starting at column lt (coalesced along the stored contiguous direction);
-  // non-finite scalars are flagged (their row's exponent becomes 0, as a non-finite maximum
-  // gives) and split as zero
-  auto load_tile = [&](int lt) {
-    // all of a thread's loads are issued before any is used, so their latencies overlap (tiles
-    // are at most 16 wide in the VEC = 2 instance, which serves K <= 16 only)
-    constexpr int NPT = SPLIT_ROWS * (VEC == 2 ? 16 : SPLIT_TK) / SPLIT_THREADS;
-    longlong2 v[NPT];
+  for (int s = p.S - 1; s >= 0; --s) {
+    uint32_t r[4], i[4], n[4];
 #pragma unroll
-    for (int u = 0; u < NPT; ++u) {
-      const int idx = tid + u * SPLIT_THREADS;
-      int rl, ll;
-      if (!p.trans) { rl = idx % SPLIT_ROWS; ll = idx / SPLIT_ROWS; }
-      else          { ll = idx % TK;         rl = idx / TK; }
-      const int r = r0 + rl, l = lt + ll;
-      v[u] = make_longlong2(0, 0);
-      if (idx < SPLIT_ROWS * TK && r < R && l < K)
-        v[u] = reinterpret_cast<const longlong2*>(P)[p.trans ? l + r * ld : r + l * ld];
-    }
-#pragma unroll
-    for (int u = 0; u < NPT; ++u) {
-      const int idx = tid + u * SPLIT_THREADS;
-      if (idx >= SPLIT_ROWS * TK) break;
-      int rl, ll;
-      if (!p.trans) { rl = idx % SPLIT_ROWS; ll = idx / SPLIT_ROWS; }
-      else          { ll = idx % TK;         rl = idx / TK; }
-      // integer operations on the bit patterns only (binary64 compares and negations would
-      // occupy this GPU's scarce FP64 pipe)
-      longlong2 w = v[u];
-      if (p.conj) w.y ^= static_cast<long long>(0x8000000000000000ull);
-      const bool fx = (w.x & 0x7FF0000000000000ll) == 0x7FF0000000000000ll;
-      const bool fy = (w.y & 0x7FF0000000000000ll) == 0x7FF0000000000000ll;
-      if (fx || fy) {
-        bad = 1;
-        rowbad[rl] = 1;
-        if (fx) w.x = 0;
-        if (fy) w.y = 0;
+    for (int q = 0; q < 8; ++q) {
+      int dr, di;
+      if constexpr (W64) {
+        dr = s ? next_digit64(Xr[q]) : static_cast<int>(Xr[q]);
+        di = s ? next_digit64(Xi[q]) : static_cast<int>(Xi[q]);
+      } else {
+        dr = s ? next_digit(Xr[q]) : static_cast<int>(Xr[q]);
+        di = s ? next_digit(Xi[q]) : static_cast<int>(Xi[q]);
       }
-      tile[rl][ll] = make_double2(__longlong_as_double(w.x), __longlong_as_double(w.y));
-    }
-  };
-
-  if (kpar) {
-    // row maxima taken by the pre-pass over all of K (a non-finite maximum flags the row)
-    if (tid < SPLIT_ROWS && r0 + tid < R) {
-      rowmax[tid] = p.gmax[z * p.exp_stride + r0 + tid];
-      if (rowmax[tid] >= 0x7FF0000000000000ull) bad = 1;
-    }
-  } else if (one_tile) {
-    load_tile(0);
-    __syncthreads();
-    // row maxima from the tile: 8 threads per row, combined by shuffles
-    const int rl = tid >> 3, cg = tid & 7;
-    unsigned long long mx = 0ull;
-    for (int l = cg; l < K; l += 8) {
-      const double2 v = tile[rl][l];
-      const unsigned long long a = static_cast<unsigned long long>(__double_as_longlong(v.x)) & 0x7FFFFFFFFFFFFFFFull;
-      const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(v.y)) & 0x7FFFFFFFFFFFFFFFull;
-      mx = max(mx, max(a, b));
-    }
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (cg == 0) rowmax[rl] = rowbad[rl] ? 0x7FF0000000000000ull : mx;
-  } else {
-    // ---- scan pass: row maxima
-    int rl, l0, lstep;
-    if (!p.trans) { rl = tid % SPLIT_ROWS; l0 = tid / SPLIT_ROWS; lstep = SPLIT_THREADS / SPLIT_ROWS; }
-    else          { rl = tid / 8;          l0 = tid % 8;          lstep = 8; }
-    const int r = r0 + rl;
-    unsigned long long mx = 0ull;
-    if (r < R) {
-      for (int l = l0; l < K; l += lstep) {
-        const double2 v = p.trans ? P[l + r * ld] : P[r + l * ld];
-        const unsigned long long a = static_cast<unsigned long long>(__double_as_longlong(v.x)) & 0x7FFFFFFFFFFFFFFFull;
-        const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(v.y)) & 0x7FFFFFFFFFFFFFFFull;
-        const unsigned long long m2 = a > b ? a : b;
-        if (m2 >= 0x7FF0000000000000ull) bad = 1;
-        mx = m2 > mx ? m2 : mx;
-      }
-      atomicMax(&rowmax[rl], mx);
-    }
-  }
-  __syncthreads();
-  if (bad && tid == 0) flag_error(p.status, OZK_ERR_NONFINITE);
-  if (tid < SPLIT_ROWS) {
-    const unsigned long long a = rowmax[tid];
-    const int e = (a >= 0x7FF0000000000000ull) ? 0 : frexp_exponent_from_bits(a);
-    rowexp[tid] = e;
-    if (r0 + tid < R && kg == 0) p.exps[z * p.exp_stride + r0 + tid] = e;
-  }
-  __syncthreads();
-
-  // ---- digits, tile by tile along K
-  const int S = p.S;
-  const long long plane = p.out_rows * p.kpad;
-  __half* outz = p.out + static_cast<long long>(z) * S * plane;
-  const bool dbg = (p.dbg_digits != nullptr) && z == 0;
-  const long long dplane = p.out_rows * 2LL * K;
-  int lt_begin = 0, lt_end = K;
-  if (kpar) {
-    const int ntk = (K + TK - 1) / TK, per_g = (ntk + kgs - 1) / kgs;
-    lt_begin = kg * per_g * TK;
-    lt_end = min(K, (kg + 1) * per_g * TK);
-  }
-  for (int lt = lt_begin; lt < lt_end; lt += TK) {
-    if (!one_tile) {
-      load_tile(lt);
-      __syncthreads();
-    }
-    // each thread: one row, 8 consecutive l
-    {
-      const int rl = tid / 8;
-      const int lg = (tid % 8) * per;
-      const int r = r0 + rl;
-      const int l0 = lt + lg;
-      // vector stores when this thread's run is whole and aligned (and no debug copy)
-      const bool vec = !dbg && ((VEC >= 8 && per == 8) || (VEC >= 4 && per == 4) || per == 2) && K % per == 0 &&
-                       l0 + per <= K;
-      if (r < R && vec) {
-        const int e = rowexp[rl];
-        if constexpr (SF > 0) {
-          if (per == 8) split_run_fixed<8, SF>(p, &tile[rl][lg], e, r, l0, K, outz, plane);
-          else if (per == 4) split_run_fixed<4, SF>(p, &tile[rl][lg], e, r, l0, K, outz, plane);
-          else split_run_fixed<2, SF>(p, &tile[rl][lg], e, r, l0, K, outz, plane);
-        } else if constexpr (VEC >= 8) {
-          if (per == 8) split_run<8, W64>(p, &tile[rl][lg], e, r, l0, K, outz, plane);
-          else if (per == 4) split_run<4, W64>(p, &tile[rl][lg], e, r, l0, K, outz, plane);
-          else split_run<2, W64>(p, &tile[rl][lg], e, r, l0, K, outz, plane);
+      const uint32_t hr = __half_as_ushort(__int2half_rn(dr)), hi = __half_as_ushort(__int2half_rn(di)),
+                     hn = __half_as_ushort(__int2half_rn(-di));
+      if (q & 1) { r[q / 2] |= hr << 16; i[q / 2] |= hi << 16; n[q / 2] |= hn << 16; }
+      else { r[q / 2] = hr; i[q / 2] = hi; n[q / 2] = hn; }
+      if (dbg && l0 + q < K) {
+        const int l = l0 + q;
+        if (SIDE == 0) {
+          int16_t* o = dbg + (static_cast<long long>(s) * p.out_rows + row) * 2LL * K;
+          o[l] = static_cast<int16_t>(dr);
+          o[K + l] = static_cast<int16_t>(di);
         } else {
-          split_run<2, W64>(p, &tile[rl][lg], e, r, l0, K, outz, plane);
-        }
-      } else if (r < R) {
-        const int e = rowexp[rl];
-        for (int q = 0; q < per; ++q) {
-          const int l = lt + lg + q;
-          if (l >= K) break;
-          const double2 v = tile[rl][lg + q];
-          __int128 Xr = integer_image(v.x, e, p.nbits);
-          __int128 Xi = integer_image(v.y, e, p.nbits);
-          // digits from the least significant (plane S-1) to the most significant (plane 0)
-          for (int s = S - 1; s >= 0; --s) {
-            const int dr = s ? next_digit(Xr) : static_cast<int>(Xr);
-            const int di = s ? next_digit(Xi) : static_cast<int>(Xi);
-            __half* o = outz + s * plane;
-            if (p.side == 0) {
-              o[r * p.kpad + l] = __int2half_rn(dr);
-              o[r * p.kpad + K + l] = __int2half_rn(di);
-              if (dbg) {
-                p.dbg_digits[s * dplane + r * 2LL * K + l] = static_cast<int16_t>(dr);
-                p.dbg_digits[s * dplane + r * 2LL * K + K + l] = static_cast<int16_t>(di);
-              }
-            } else {
-              const long long row0 = 2LL * r, row1 = 2LL * r + 1;
-              o[row0 * p.kpad + l] = __int2half_rn(dr);
-              o[row0 * p.kpad + K + l] = __int2half_rn(-di);
-              o[row1 * p.kpad + l] = __int2half_rn(di);
-              o[row1 * p.kpad + K + l] = __int2half_rn(dr);
-              if (dbg) {
-                p.dbg_digits[s * dplane + row0 * 2LL * K + l] = static_cast<int16_t>(dr);
-                p.dbg_digits[s * dplane + row0 * 2LL * K + K + l] = static_cast<int16_t>(-di);
-                p.dbg_digits[s * dplane + row1 * 2LL * K + l] = static_cast<int16_t>(di);
-                p.dbg_digits[s * dplane + row1 * 2LL * K + K + l] = static_cast<int16_t>(dr);
-              }
-            }
-          }
+          int16_t* o = dbg + (static_cast<long long>(s) * p.out_rows + 2LL * row) * 2LL * K;
+          o[l] = static_cast<int16_t>(dr);
+          o[K + l] = static_cast<int16_t>(-di);
+          o[2LL * K + l] = static_cast<int16_t>(di);
+          o[3LL * K + l] = static_cast<int16_t>(dr);
         }
       }
     }
-    __syncthreads();
-  }
-  // zero the K padding [2K, kpad) of the rows this CTA owns (one CTA of a row block)
-  const int pad = static_cast<int>(p.kpad) - 2 * K;
-  if (pad > 0 && kg == kgs - 1) {
-    const int rows_out = p.side == 0 ? 1 : 2;
-    const int nr = min(SPLIT_ROWS, R - r0) * rows_out;
-    for (int idx = tid; idx < S * nr * pad; idx += SPLIT_THREADS) {
-      const int c = idx % pad;
-      const int rr = (idx / pad) % nr;
-      const int s = idx / (pad * nr);
-      outz[s * plane + (static_cast<long long>(r0) * rows_out + rr) * p.kpad + 2 * K + c] = __float2half(0.0f);
-    }
+    store_slice(d, s, r, i, n);
   }
 }
 
-// Row maxima for the K-parallel split: CTA x covers 32 rows (x / nseg) and K segment x % nseg
-// of SPLIT_KSEG elements; each row's largest |Re|, |Im| bit pattern (non-finite values compare
-// above every finite one) reaches gmax by one 64-bit atomicMax per row and CTA.
-constexpr int SPLIT_KSEG = 512;
-__global__ void __launch_bounds__(SPLIT_THREADS) split_rowmax_kernel(const SplitPair pp, int nseg) {
-  if (static_cast<int>(blockIdx.z) >= pp.nsides) return;
-  const SplitParams& p = pp.s[blockIdx.z];
-  if (!p.gmax) return;
+__device__ __forceinline__ unsigned long long abs_bits(long long x) {
+  return static_cast<unsigned long long>(x) & 0x7FFFFFFFFFFFFFFFull;
+}
+
+// 8 elements (zero past K) of logical row r from element l0 on; trans: they are contiguous
+__device__ __forceinline__ void load_block(const SplitParams& p, const longlong2* __restrict__ P, long long ld, int r,
+                                           int l0, int K, longlong2 (&v)[8]) {
+  const longlong2* s = P + (p.trans ? l0 + r * ld : r + l0 * ld);
+  const long long step = p.trans ? 1 : ld;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) v[q] = l0 + q < K ? s[q * step] : make_longlong2(0, 0);
+}
+
+// largest |Re|, |Im| bit pattern (non-finite values compare above every finite one)
+__device__ __forceinline__ unsigned long long block_max(const longlong2 (&v)[8]) {
+  unsigned long long mx = 0ull;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) mx = max(mx, max(abs_bits(v[q].x), abs_bits(v[q].y)));
+  return mx;
+}
+
+// Both operands of one emulated GEMM in one launch: blockIdx.z selects the side.  A CTA owns 32
+// rows, one per lane; warp w takes the K-blocks w, w + nwarps, ... of its share.  With kgroups > 1
+// the CTAs of a cluster share a row block's K-blocks and exchange their row maxima through
+// distributed shared memory.  A share of at most one K-block per warp is read from memory once and
+// kept in registers between the maximum and the digits; longer shares are read twice.  Non-finite
+// scalars flag OZK_ERR_NONFINITE, make their row's exponent 0 and are split as zero.
+template <int SF, bool W64, int SIDE>
+__device__ __forceinline__ void split_rows(const SplitParams& p, unsigned long long (&wmax)[SPLIT_MAX_WARPS][SPLIT_ROWS],
+                                           unsigned long long (&cmax)[SPLIT_MAX_KG][SPLIT_ROWS]) {
   const int z = blockIdx.y;
   const bool single = p.X == nullptr;
   const int R = single ? p.rows1 : p.rows[z];
   const int K = single ? p.k1 : p.kdim[z];
-  const int r0 = (static_cast<int>(blockIdx.x) / nseg) * SPLIT_ROWS;
-  const int l_lo = (static_cast<int>(blockIdx.x) % nseg) * SPLIT_KSEG;
-  if (r0 >= R || l_lo >= K) return;
-  const int l_hi = min(K, l_lo + SPLIT_KSEG);
-  const double2* __restrict__ P = single ? p.X1 + z * p.zstride1 : p.X[z];
+  const int kgs = p.kgroups;
+  const int rank = static_cast<int>(blockIdx.x) % kgs;
+  const int r0 = (static_cast<int>(blockIdx.x) / kgs) * SPLIT_ROWS;
+  if (r0 >= R) return;                                 // the same for every CTA of the cluster
+  if (kgs > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  const longlong2* __restrict__ P = reinterpret_cast<const longlong2*>(single ? p.X1 + z * p.zstride1 : p.X[z]);
   const long long ld = single ? p.ld1 : p.ld[z];
-  __shared__ unsigned long long mx_s[SPLIT_ROWS];
-  const int tid = threadIdx.x;
-  if (tid < SPLIT_ROWS) mx_s[tid] = 0ull;
-  __syncthreads();
-  int rl, l0, lstep;
-  if (!p.trans) { rl = tid % SPLIT_ROWS; l0 = tid / SPLIT_ROWS; lstep = SPLIT_THREADS / SPLIT_ROWS; }
-  else          { rl = tid / 8;          l0 = tid % 8;          lstep = 8; }
-  const int r = r0 + rl;
-  if (r < R) {
-    unsigned long long mx = 0ull;
-    for (int l = l_lo + l0; l < l_hi; l += lstep) {
-      const double2 v = p.trans ? P[l + r * ld] : P[r + l * ld];
-      const unsigned long long a = static_cast<unsigned long long>(__double_as_longlong(v.x)) & 0x7FFFFFFFFFFFFFFFull;
-      const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(v.y)) & 0x7FFFFFFFFFFFFFFFull;
-      mx = max(mx, max(a, b));
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int r = r0 + lane;
+  const bool rok = r < R;
+  const int nkb = (K + 7) >> 3, share = (nkb + kgs - 1) / kgs;
+  const int kb0 = rank * share, kb1 = min(nkb, kb0 + share);
+  const bool resident = share <= nw;
+
+  longlong2 v[8];
+  unsigned long long mx = 0ull;
+  if (rok) {
+    if (resident) {
+      if (kb0 + warp < kb1) {
+        load_block(p, P, ld, r, 8 * (kb0 + warp), K, v);
+        mx = block_max(v);
+      }
+    } else {
+      for (int kb = kb0 + warp; kb < kb1; kb += nw) {
+        load_block(p, P, ld, r, 8 * kb, K, v);
+        mx = max(mx, block_max(v));
+      }
     }
-    atomicMax(&mx_s[rl], mx);
   }
+  wmax[warp][lane] = mx;
   __syncthreads();
-  if (tid < SPLIT_ROWS && r0 + tid < R) atomicMax(&p.gmax[z * p.exp_stride + r0 + tid], mx_s[tid]);
+  for (int w = 0; w < nw; ++w) mx = max(mx, wmax[w][lane]);
+  if (kgs > 1) {
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");      // every peer has started
+    if (warp < kgs) {
+      uint32_t dst;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(smem_u32(&cmax[rank][lane])), "r"(warp));
+      asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(dst), "l"(mx) : "memory");
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    for (int c = 0; c < kgs; ++c) mx = max(mx, cmax[c][lane]);
+  }
+  const bool bad = mx >= 0x7FF0000000000000ull;
+  const int e = bad ? 0 : frexp_exponent_from_bits(mx);
+  if (warp == 0 && rank == 0 && rok) {
+    if (bad) flag_error(p.status, OZK_ERR_NONFINITE);
+    p.exps[z * p.exp_stride + r] = e;
+  }
+  if (!rok) return;
+
+  const int halves = static_cast<int>(p.kpad >> 3);    // halves of a plane
+  SplitDst<SIDE> d;
+  d.splane = static_cast<int>(p.out_rows);
+  d.hplane = static_cast<long long>(p.S) * p.out_rows;
+  uint4* outz = reinterpret_cast<uint4*>(p.out) + static_cast<long long>(z) * halves * d.hplane;
+  for (int kb = kb0 + warp; kb < kb1; kb += nw) {
+    if (!resident) load_block(p, P, ld, r, 8 * kb, K, v);
+    if (p.conj) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q].y ^= static_cast<long long>(0x8000000000000000ull);
+    }
+    if (bad) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        if (abs_bits(v[q].x) >= 0x7FF0000000000000ull) v[q].x = 0;
+        if (abs_bits(v[q].y) >= 0x7FF0000000000000ull) v[q].y = 0;
+      }
+    }
+    d.out = outz + 2LL * kb * d.hplane + (SIDE == 0 ? r : 2 * r);
+    d.tail4 = K - 8 * kb <= 4;
+    d.has2 = 2 * kb + 1 < halves;
+    if constexpr (SF > 0) emit_fixed<SF, SIDE>(d, v, e);
+    else emit_generic<W64, SIDE>(p, d, v, e, r, 8 * kb, K, z == 0 ? p.dbg_digits : nullptr);
+  }
+}
+
+template <int SF, bool W64>
+__global__ void __launch_bounds__(SPLIT_MAX_WARPS * 32, 2) split_kernel(const __grid_constant__ SplitPair pp) {
+  __shared__ unsigned long long wmax[SPLIT_MAX_WARPS][SPLIT_ROWS];     // row maxima of the warps
+  __shared__ unsigned long long cmax[SPLIT_MAX_KG][SPLIT_ROWS];        // and of the cluster's CTAs
+  if (pp.s[blockIdx.z].side == 0) split_rows<SF, W64, 0>(pp.s[blockIdx.z], wmax, cmax);
+  else split_rows<SF, W64, 1>(pp.s[blockIdx.z], wmax, cmax);
 }
 
 void launch_split(const SplitParams& a, int rows_a, const SplitParams* b, int rows_b, int kmax, int batch,
@@ -461,43 +350,43 @@ void launch_split(const SplitParams& a, int rows_a, const SplitParams* b, int ro
   if (b) pp.s[1] = *b;
   const int rows = std::max(rows_a, b ? rows_b : 0);
   const int rblocks = (rows + SPLIT_ROWS - 1) / SPLIT_ROWS;
-  // few row blocks and rows longer than one tile: share each row block's K tiles among kgroups
-  // CTAs, after a pre-pass that takes the row maxima over K segments
-  int kgroups = 1;
-  const bool can_kpar = pp.s[0].gmax && (pp.nsides < 2 || pp.s[1].gmax);
-  if (can_kpar && kmax > SPLIT_TK) {
-    const long long ctas = static_cast<long long>(rblocks) * batch * pp.nsides;
-    const int sms = gpu_sm_count();
-    if (ctas < sms) {
-      const int ntk = (kmax + SPLIT_TK - 1) / SPLIT_TK;
-      kgroups = static_cast<int>(std::min<long long>(ntk, std::max<long long>(1, (2LL * sms) / ctas)));
-    }
-  }
-  for (int sd = 0; sd < pp.nsides; ++sd) pp.s[sd].kgroups = kgroups;
-  if (kgroups > 1) {
-    const int nseg = (kmax + SPLIT_KSEG - 1) / SPLIT_KSEG;
-    for (int sd = 0; sd < pp.nsides; ++sd)
-      cudaMemsetAsync(pp.s[sd].gmax, 0, sizeof(unsigned long long) * pp.s[sd].exp_stride * batch, st);
-    split_rowmax_kernel<<<dim3(rblocks * nseg, batch, pp.nsides), SPLIT_THREADS, 0, st>>>(pp, nseg);
-    record_launch();
-  }
-  dim3 grid(rblocks * kgroups, batch, pp.nsides);
-  const bool w64 = pp.s[0].nbits <= 62 && (pp.nsides < 2 || pp.s[1].nbits <= 62);
-  if (kmax <= 16) {
-    if (w64) split_kernel<2, true><<<grid, SPLIT_THREADS, 0, st>>>(pp);
-    else split_kernel<2, false><<<grid, SPLIT_THREADS, 0, st>>>(pp);
-  } else {
-    // compile-time slice counts for the common S = 7 and S = 5 (nbits = 8 S - 1 on every side)
-    int sf = 0;
-    for (int S : {7, 5}) {
-      bool all = true;
-      for (int sd = 0; sd < pp.nsides; ++sd) all = all && pp.s[sd].S == S && pp.s[sd].nbits == 8 * S - 1;
-      if (all) { sf = S; break; }
-    }
-    if (sf == 7) split_kernel<8, true, 7><<<grid, SPLIT_THREADS, 0, st>>>(pp);
-    else if (sf == 5) split_kernel<8, true, 5><<<grid, SPLIT_THREADS, 0, st>>>(pp);
-    else if (w64) split_kernel<8, true><<<grid, SPLIT_THREADS, 0, st>>>(pp);
-    else split_kernel<8, false><<<grid, SPLIT_THREADS, 0, st>>>(pp);
+  const int nkb = (kmax + 7) / 8;
+  // a cluster of up to 8 CTAs shares a row block's K-blocks when its rows are longer than the 8
+  // K-blocks that a CTA reads once (K > 64), or while the launch has fewer than two CTAs per SM
+  // and a CTA would keep at least 8 K-blocks
+  const long long ctas = static_cast<long long>(rblocks) * batch * pp.nsides;
+  int kg = 1;
+  while (kg < SPLIT_MAX_KG && ((nkb + kg - 1) / kg > SPLIT_MAX_WARPS ||
+                               (ctas * kg < 2LL * gpu_sm_count() && nkb / (2 * kg) >= 8)))
+    kg *= 2;
+  const int share = (nkb + kg - 1) / kg;
+  for (int sd = 0; sd < pp.nsides; ++sd) pp.s[sd].kgroups = kg;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(rblocks * kg), static_cast<unsigned>(batch), static_cast<unsigned>(pp.nsides));
+  cfg.blockDim = dim3(32u * static_cast<unsigned>(std::max(std::min(share, SPLIT_MAX_WARPS), kg)));
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = static_cast<unsigned>(kg);
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = kg > 1 ? 1 : 0;
+  // compile-time slice counts 3..8 (nbits = 8 S - 1 on every side); the test hook's digit copy and
+  // other slice counts take the run-time form
+  int sf = pp.s[0].S;
+  for (int sd = 0; sd < pp.nsides; ++sd)
+    if (pp.s[sd].S != sf || pp.s[sd].nbits != 8 * sf - 1 || pp.s[sd].dbg_digits) sf = 0;
+  switch (sf) {
+    case 3: cudaLaunchKernelEx(&cfg, split_kernel<3, true>, pp); break;
+    case 4: cudaLaunchKernelEx(&cfg, split_kernel<4, true>, pp); break;
+    case 5: cudaLaunchKernelEx(&cfg, split_kernel<5, true>, pp); break;
+    case 6: cudaLaunchKernelEx(&cfg, split_kernel<6, true>, pp); break;
+    case 7: cudaLaunchKernelEx(&cfg, split_kernel<7, true>, pp); break;
+    case 8: cudaLaunchKernelEx(&cfg, split_kernel<8, true>, pp); break;
+    default:
+      if (pp.s[0].nbits <= 62 && (pp.nsides < 2 || pp.s[1].nbits <= 62)) cudaLaunchKernelEx(&cfg, split_kernel<0, true>, pp);
+      else cudaLaunchKernelEx(&cfg, split_kernel<0, false>, pp);
   }
   record_launch();
 }
