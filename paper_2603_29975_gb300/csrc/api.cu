@@ -278,7 +278,7 @@ struct EmuGemm {
 };
 
 struct GemmPlan {
-  int G, BN, maxpairs, npairs, kpad, rowsA, rowsB, nstage, chunk_kb, kblocks, magic;
+  int G, BN, maxpairs, npairs, kpad, rowsA, rowsB, chunk_kb, kblocks, magic;
   int ksplit;                                 // split-K units per tile (single problems with few tiles)
   size_t offA, offB, offE, offF, offT, offP, offGA, offGB, total;
 };
@@ -297,9 +297,7 @@ ozk_status_t plan_gemm(const EmuGemm& g, GemmPlan* P) {
   P->kpad = static_cast<int>(align_up(static_cast<size_t>(std::max<long long>(kp2, 16)), 8));
   P->rowsA = std::max(g.mmax, 1);
   P->rowsB = 2 * std::max(g.nmax, 1);
-  const size_t stage = static_cast<size_t>(S) * (128 + P->BN) * 32;
-  P->nstage = static_cast<int>(std::min<size_t>(6, (227 * 1024 - 14 * 1024) / stage));
-  if (P->nstage < 1) return set_error(OZK_ERR_ARG, "S too large for the shared-memory pipeline");
+  if (gemm_stages(S, P->BN) < 1) return set_error(OZK_ERR_ARG, "S too large for the shared-memory pipeline");
   P->kblocks = static_cast<int>((kp2 + 15) / 16);
   // exactness chunk: every product of two digits is <= 2^14 in magnitude; an FP32 accumulator
   // stays exact up to 2^24 (1024 terms) and allows the one-add conversion below 2^22 (255 terms)
@@ -409,7 +407,7 @@ ozk_status_t run_emulated(ozk_context* h, const EmuGemm& g, size_t ws_offset = 0
   if (st) return st;
 
   GemmParams gp{};
-  gp.S = S; gp.ngroups = P.G; gp.kblocks = P.kblocks; gp.chunk_kb = P.chunk_kb; gp.nstage = P.nstage;
+  gp.S = S; gp.ngroups = P.G; gp.kblocks = P.kblocks; gp.chunk_kb = P.chunk_kb;
   gp.magic = P.magic;
   {
     // group g receives the products of its own pairs only: 16 per K-block and pair, each at most
@@ -446,6 +444,7 @@ ozk_status_t run_emulated(ozk_context* h, const EmuGemm& g, size_t ws_offset = 0
   else if (g.br == 0.0 && g.bi == 0.0) gp.mode = 0;
   else if (g.ar == -1.0 && g.ai == 0.0 && g.br == 1.0 && g.bi == 0.0) gp.mode = 1;
   else gp.mode = 2;
+  gp.nstage = gemm_stages(S, P.BN);
   gp.e = e; gp.f = f; gp.e_stride = P.rowsA; gp.f_stride = std::max(g.nmax, 1);
   gp.groups = g.groups; gp.status = h->d_status;
   if (single) { gp.m = nullptr; gp.m1 = g.m; gp.n1 = g.n; gp.C1 = g.C; gp.ldc1 = g.ldc; gp.skm1 = g.skm; gp.skn1 = g.skn; }

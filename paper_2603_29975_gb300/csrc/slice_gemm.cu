@@ -7,10 +7,16 @@
 
 namespace ozk {
 
-size_t gemm_smem_bytes(int S, int BN, int nstage) {
+static size_t gemm_smem_bytes(int S, int BN, int nstage) {
   const size_t stage = static_cast<size_t>(S) * (GEMM_BM + BN) * 32;
   const size_t ring = GEMM_TILE_SLOTS * (BN == 64 ? sizeof(TileInfo<64>) : sizeof(TileInfo<32>));
   return 1024 + nstage * stage + ring + (2 * nstage + 20 + 2 * GEMM_TILE_SLOTS) * 8 + 16;
+}
+
+int gemm_stages(int S, int BN) {
+  int n = 6;
+  while (n > 0 && gemm_smem_bytes(S, BN, n) > 227 * 1024) --n;
+  return n;
 }
 
 static int num_sms() {

@@ -366,10 +366,6 @@ __device__ __forceinline__ RowInfo out_row(const GemmParams& p, bool single, int
   return o;
 }
 
-__device__ __forceinline__ void prefetch_l2(const void* ptr) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<uint64_t>(ptr)));
-}
-
 // Waits of the epilogue for the accumulators of one tile: its exactness chunks complete one after
 // the other, each in two parts (acc_full; chunk counter cc, running over the CTA's tiles).
 struct ChunkWait {
@@ -496,40 +492,19 @@ __device__ __forceinline__ bool fold_part(const EpiCtx& x, uint64_t* acc_empty, 
   return true;
 }
 
-// One complex output: z rounded (EPI_IMINUS: -Z rounded), c the old value of C.
-__device__ __forceinline__ void combine_one(const GemmParams& p, double2* d, double zr, double zi, double2 c, bool diag) {
-  if (p.mode == EPI_LU) {
-    *d = make_double2(c.x - zr, c.y - zi);
-  } else if (p.mode == EPI_IMINUS) {
-    *d = make_double2(diag ? 1.0 + zr : zr, zi);          // off the diagonal 0 - RN(Z) = RN(-Z)
-  } else if (p.mode == EPI_STORE && p.unit_alpha) {
-    *d = make_double2(zr, zi);
-  } else {
-    double xr = p.ar * zr - p.ai * zi, xi = p.ar * zi + p.ai * zr;
-    if (p.mode != EPI_STORE) {
-      xr = xr + (p.br * c.x - p.bi * c.y);
-      xi = xi + (p.br * c.y + p.bi * c.x);
-    }
-    *d = make_double2(xr, xi);
-  }
-}
-
-// Four complex outputs of a row (columns jc .. jc + 3 at d, d + ld, ...); ok: which are written.  The
-// mode is tested once for the four, and the stores of one mode follow each other.
-__device__ __forceinline__ void combine_store(const GemmParams& p, double2* d, long long ld, int jc, int grow,
-                                              const bool (&ok)[4], const double (&z)[8], const double2 (&cv)[4]) {
-  if (p.mode == EPI_LU) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q, d += ld)
-      if (ok[q]) *d = make_double2(cv[q].x - z[2 * q], cv[q].y - z[2 * q + 1]);
-  } else if (p.mode == EPI_STORE && p.unit_alpha) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q, d += ld)
-      if (ok[q]) *d = make_double2(z[2 * q], z[2 * q + 1]);
-  } else {
-#pragma unroll
-    for (int q = 0; q < 4; ++q, d += ld)
-      if (ok[q]) combine_one(p, d, z[2 * q], z[2 * q + 1], cv[q], jc + q == grow);
+// One complex output: (zr, zi), z rounded (EPI_IMINUS: -Z rounded), becomes the value to store; c the
+// old value of C (UPDATE).
+template <bool UPDATE>
+__device__ __forceinline__ void combine(const GemmParams& p, double& zr, double& zi, double2 c, bool diag) {
+  if (UPDATE && p.mode == EPI_LU) {
+    zr = c.x - zr;
+    zi = c.y - zi;
+  } else if (!UPDATE && p.mode == EPI_IMINUS) {
+    if (diag) zr = 1.0 + zr;                              // off the diagonal 0 - RN(Z) = RN(-Z)
+  } else if (UPDATE || !p.unit_alpha) {
+    const double xr = p.ar * zr - p.ai * zi, xi = p.ar * zi + p.ai * zr;
+    zr = UPDATE ? xr + (p.br * c.x - p.bi * c.y) : xr;
+    zi = UPDATE ? xi + (p.br * c.y + p.bi * c.x) : xi;
   }
 }
 
@@ -540,19 +515,35 @@ __device__ __forceinline__ void combine_store(const GemmParams& p, double2* d, l
 // chunk).  A thread owns one row and 16 stacked columns (8 complex).  The groups are read two at a
 // time and released as soon as they are read, so the MMAs of the next chunk or tile start while
 // the rest is folded, rounded and written.  The outputs are rounded and combined in two halves of
-// 4 complex columns, the second half's C values requested before the first half is combined.
+// 4 complex columns.
 // Returns false if a wait gave up.
-template <int G, bool F64, bool KS = false>
+// UPDATE: the mode combines with C (a separate instance: the values' registers would spill the others).
+template <int G, bool F64, bool KS, bool UPDATE>
 __device__ __forceinline__ bool epilogue_fast(const GemmParams& p, const EpiCtx& x, uint64_t* acc_empty,
                                               uint32_t magic_mask, int lane, ChunkWait& cw) {
   constexpr int NH = F64 ? G : (G < 4 ? G : 4);
   constexpr int NL = G - NH;
   constexpr int S8 = 8 * NL;
-  const bool needC = p.mode == EPI_LU || p.mode == EPI_GENERAL;
   const int jc0 = (x.n0 + x.c0) / 2;                  // this thread's 8 complex columns
   const int jend = min(min(jc0 + 8, (x.n2 + 1) / 2), x.jlim);
   const bool active = x.rowok && max(jc0, x.skip_n) < jend;
   if (!__any_sync(0xffffffffu, active)) return release_unread<G>(acc_empty, cw, lane);
+  double2* Cp = x.C + jc0 * x.ld;
+  auto wanted = [&](int jj) { return active && jc0 + jj < jend && jc0 + jj >= x.skip_n; };
+  // C's values go straight to registers, requested when those of the sums' halves become free: copies
+  // into shared memory (cp.async, by the threads themselves or by a warp of its own) arrive only after
+  // 4 to 8 us beside the tensor pipe's operand reads, and values requested before the drain spill the
+  // sums
+  auto load_c = [&](int half, double2 (&cv)[4]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      cv[q] = UPDATE && wanted(4 * half + q) ? Cp[(4 * half + q) * x.ld] : make_double2(0.0, 0.0);
+  };
+  if constexpr (UPDATE) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if (wanted(q)) asm volatile("prefetch.global.L2 [%0];" ::"l"(Cp + q * x.ld));
+  }
   unsigned long long H[16], L[16];
   const unsigned long long bh = 0ull - static_cast<unsigned long long>(cw.nchunks) * FoldPlan<G, NH>::bias(0, NH);
   const unsigned long long bl = 0ull - static_cast<unsigned long long>(cw.nchunks) * FoldPlan<G, NH>::bias(NH, G);
@@ -577,9 +568,8 @@ __device__ __forceinline__ bool epilogue_fast(const GemmParams& p, const EpiCtx&
     }
     return true;
   }
-  const bool neg = p.mode == EPI_IMINUS;
+  const bool neg = !UPDATE && p.mode == EPI_IMINUS;
   const int* f = x.f + x.c0 / 2;                      // (zero past the problem's columns)
-  double2* Cp = x.C + jc0 * x.ld;
   bool near = exponent_near(x.er);
 #pragma unroll
   for (int jj = 0; jj < 8; ++jj) near = near && exponent_near(f[jj]);
@@ -592,24 +582,16 @@ __device__ __forceinline__ bool epilogue_fast(const GemmParams& p, const EpiCtx&
       for (int q = 0; q < 8; ++q)
         if (q == jj) { hr = H[2 * q]; lr = L[2 * q]; hi = H[2 * q + 1]; li = L[2 * q + 1]; }
       const int E = x.er + f[jj], jc = jc0 + jj;
-      const double zr = round_far(static_cast<long long>(neg ? 0ull - hr : hr), static_cast<long long>(neg ? 0ull - lr : lr), S8, E);
-      const double zi = round_far(static_cast<long long>(neg ? 0ull - hi : hi), static_cast<long long>(neg ? 0ull - li : li), S8, E);
-      if (active && jc < jend && jc >= x.skip_n)
-        combine_one(p, Cp + jj * x.ld, zr, zi, needC ? Cp[jj * x.ld] : make_double2(0.0, 0.0), jc == x.grow);
+      double zr = round_far(static_cast<long long>(neg ? 0ull - hr : hr), static_cast<long long>(neg ? 0ull - lr : lr), S8, E);
+      double zi = round_far(static_cast<long long>(neg ? 0ull - hi : hi), static_cast<long long>(neg ? 0ull - li : li), S8, E);
+      if (!wanted(jj)) continue;
+      combine<UPDATE>(p, zr, zi, UPDATE ? Cp[jj * x.ld] : make_double2(0.0, 0.0), jc == x.grow);
+      Cp[jj * x.ld] = make_double2(zr, zi);
     }
     return true;
   }
-  auto outputs_ok = [&](int half, bool (&ok)[4]) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int jc = jc0 + 4 * half + q;
-      ok[q] = active && jc < jend && jc >= x.skip_n;
-    }
-  };
-  auto load_c = [&](int half, const bool (&ok)[4], double2 (&cv)[4]) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) cv[q] = (needC && ok[q]) ? Cp[(4 * half + q) * x.ld] : make_double2(0.0, 0.0);
-  };
+  // the first half's subtractions (FP64 pipe) stand before the second half's roundings (integer
+  // pipes), and its stores after them, so that the two can overlap
   auto round_half = [&](int half, double (&z)[8]) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -618,17 +600,27 @@ __device__ __forceinline__ bool epilogue_fast(const GemmParams& p, const EpiCtx&
       for (int h = 0; h < 2; ++h) z[2 * q + h] = round_hl<S8>(H[8 * half + 2 * q + h], L[8 * half + 2 * q + h], ehi);
     }
   };
-  bool ok0[4], ok1[4];
-  double2 c0[4], c1[4];
+  auto combine_half = [&](int half, double (&z)[8], const double2 (&cv)[4]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) combine<UPDATE>(p, z[2 * q], z[2 * q + 1], cv[q], jc0 + 4 * half + q == x.grow);
+  };
+  auto store_half = [&](int half, const double (&z)[8]) {
+    double2* d = Cp + 4 * half * x.ld;
+#pragma unroll
+    for (int q = 0; q < 4; ++q, d += x.ld) {
+      if (wanted(4 * half + q)) *d = make_double2(z[2 * q], z[2 * q + 1]);
+    }
+  };
   double z0[8], z1[8];
-  outputs_ok(0, ok0);
-  load_c(0, ok0, c0);
+  double2 c0[4], c1[4];
+  load_c(0, c0);
   round_half(0, z0);
-  outputs_ok(1, ok1);
-  load_c(1, ok1, c1);
-  combine_store(p, Cp, x.ld, jc0, x.grow, ok0, z0, c0);
+  combine_half(0, z0, c0);
+  load_c(1, c1);
   round_half(1, z1);
-  combine_store(p, Cp + 4 * x.ld, x.ld, jc0 + 4, x.grow, ok1, z1, c1);
+  store_half(0, z0);
+  combine_half(1, z1, c1);
+  store_half(1, z1);
   return true;
 }
 
@@ -675,8 +667,8 @@ slice_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     for (int i = 0; i < 16; ++i) mbar_init(&acc_empty[i], GEMM_EPI_WARPS);
     mbar_init(done_bar, 1);
     mbar_init(stall_bar, 1);
-    // a slot's readers: the TMA, MMA and prefetch warps and the epilogue warps
-    for (int i = 0; i < GEMM_TILE_SLOTS; ++i) { mbar_init(&tile_full[i], 1); mbar_init(&tile_empty[i], 3 + GEMM_EPI_WARPS); }
+    // a slot's readers: the TMA and MMA threads and the epilogue warps
+    for (int i = 0; i < GEMM_TILE_SLOTS; ++i) { mbar_init(&tile_full[i], 1); mbar_init(&tile_empty[i], 2 + GEMM_EPI_WARPS); }
     *abort_flag = 0;
     mbar_fence_init();
     prefetch_tensormap(&tmA);
@@ -938,24 +930,6 @@ slice_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         ++i;
         if (end) break;
       }
-    } else {
-      // ---------------- prefetch warp: the tile's C towards L2 (updates only)
-      const bool needC = p.mode == EPI_LU || p.mode == EPI_GENERAL;
-      for (uint32_t i = 0; !stalled; ++i) {
-        int got = lane == 0 ? (tile_at(i) != nullptr) : 0;
-        if (!__shfl_sync(0xffffffffu, got, 0)) break;
-        const TileInfo<BN>* ti = ring + i % GEMM_TILE_SLOTS;
-        if (ti->end) break;
-        if (needC) {
-          // 8 rows of 16 bytes to a 128-byte line: 16 lanes for the rows of a column, 2 columns a step
-          const RowInfo o = ti->row[8 * (lane & 15)];
-          const int j0 = ti->n0 / 2, j1 = min(j0 + BN / 2, ti->n2 / 2);
-          if (o.C)
-            for (int j = j0 + (lane >> 4); j < j1; j += 2) prefetch_l2(o.C + static_cast<long long>(j) * o.ld);
-        }
-        __syncwarp();
-        if (lane == 0) tile_done(i);
-      }
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(GEMM_EPI_REGS));
@@ -965,6 +939,7 @@ slice_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     const int c0 = slab * COLS;                  // first local stacked column of this thread
     const uint32_t tbase = tmem + (static_cast<uint32_t>(quad * 32) << 16) + c0;
     const bool magic = p.magic != 0;
+    const bool update = p.mode == EPI_LU || p.mode == EPI_GENERAL;
     const uint32_t magic_mask = magic ? 0xFFFFFFFFu : static_cast<uint32_t>(p.magic_mask);
     uint32_t cc = 0;
     bool ok = !stalled;
@@ -987,18 +962,29 @@ slice_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           x.f = ti->f;
           ChunkWait cw{acc_full, unch, &cc, p.status, abort_flag};
           bool e_ok;
-          if constexpr (SF > 0) {
-            if (SF <= 5 && p.fit64) e_ok = epilogue_fast<SF, (SF <= 5)>(p, x, acc_empty, magic_mask, lane, cw);
-            else e_ok = epilogue_fast<SF, false, KS>(p, x, acc_empty, magic_mask, lane, cw);
+          if constexpr (KS) {
+            // (a split K's sums are combined by the finishing kernel)
+#define OZK_EPI(GG) case GG: e_ok = epilogue_fast<GG, false, true, false>(p, x, acc_empty, magic_mask, lane, cw); break
+            if constexpr (SF > 0) {
+              switch (SF) { OZK_EPI(SF); default: e_ok = false; }
+            } else {
+              switch (G) { OZK_EPI(1); OZK_EPI(2); OZK_EPI(3); OZK_EPI(4); OZK_EPI(5); OZK_EPI(6); OZK_EPI(7); OZK_EPI(8); default: e_ok = false; }
+            }
+#undef OZK_EPI
           } else {
 #define OZK_EPI(GG) \
   case GG: \
-    e_ok = (GG <= 5 && p.fit64) ? epilogue_fast<GG, (GG <= 5)>(p, x, acc_empty, magic_mask, lane, cw) \
-                                : epilogue_fast<GG, false, KS>(p, x, acc_empty, magic_mask, lane, cw); \
+    if (GG <= 5 && p.fit64) \
+      e_ok = update ? epilogue_fast<GG, (GG <= 5), false, true>(p, x, acc_empty, magic_mask, lane, cw) \
+                    : epilogue_fast<GG, (GG <= 5), false, false>(p, x, acc_empty, magic_mask, lane, cw); \
+    else \
+      e_ok = update ? epilogue_fast<GG, false, false, true>(p, x, acc_empty, magic_mask, lane, cw) \
+                    : epilogue_fast<GG, false, false, false>(p, x, acc_empty, magic_mask, lane, cw); \
     break
-            switch (G) {
-              OZK_EPI(1); OZK_EPI(2); OZK_EPI(3); OZK_EPI(4); OZK_EPI(5); OZK_EPI(6); OZK_EPI(7);
-              default: e_ok = epilogue_fast<8, false, KS>(p, x, acc_empty, magic_mask, lane, cw); break;
+            if constexpr (SF > 0) {
+              switch (SF) { OZK_EPI(SF); default: e_ok = false; }
+            } else {
+              switch (G) { OZK_EPI(1); OZK_EPI(2); OZK_EPI(3); OZK_EPI(4); OZK_EPI(5); OZK_EPI(6); OZK_EPI(7); OZK_EPI(8); default: e_ok = false; }
             }
 #undef OZK_EPI
           }
@@ -1073,8 +1059,10 @@ slice_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             if (2 * jc < n2_z && jc >= skip_n && jc < jlim) {
               const int E = ti->e[rl] + ti->f[(c0 + j) >> 1];
               double2* dst = o.C + static_cast<long long>(jc) * o.ld;
-              combine_one(p, dst, round_scaled_dev(neg ? -T[j] : T[j], E), round_scaled_dev(neg ? -T[j + 1] : T[j + 1], E),
-                          needC ? *dst : make_double2(0.0, 0.0), jc == o.grow);
+              double zr = round_scaled_dev(neg ? -T[j] : T[j], E), zi = round_scaled_dev(neg ? -T[j + 1] : T[j + 1], E);
+              if (needC) combine<true>(p, zr, zi, *dst, false);
+              else combine<false>(p, zr, zi, make_double2(0.0, 0.0), jc == o.grow);
+              *dst = make_double2(zr, zi);
             }
           }
         }
