@@ -334,7 +334,7 @@ gjinv_kernel(const GjParams p, int skip_lo, int skip_hi) {
 // w^3 complex multiply-adds per block, as in gjinv_kernel; 350 against 423 us per 64 x 64
 // block on one SM.  Its 128 registers a thread fill half of an SM's register file, so two
 // such CTAs on one SM leave no room for the side stream's split CTAs that run beside the
-// shared-memory kernel: it serves launches of at most one block per SM.  Rows at or beyond w
+// shared-memory kernel: it serves launches of at most one block per SM that are too many for clusters.  Rows at or beyond w
 // are skipped, but a warp spans 32 columns whatever w is, so narrower blocks (w = 48: 3/4 of
 // the lanes busy) stay with the shared-memory kernel.
 constexpr int GJR_THREADS = 256;
@@ -460,6 +460,214 @@ gjinv_reg_kernel(const GjParams p) {
       if (i < w) xo[i] = singular ? make_double2(0.0, 0.0) : a[c];
     }
   }
+}
+
+// The same Gauss-Jordan inversion with each block spread over a cluster of C CTAs (2, 4 or 8): CTA c
+// keeps the columns c, c + C, ... of its block in shared memory.  A step needs column k (after the
+// exchange, its multipliers), the pivot's row and its reciprocal in every CTA, everything else is
+// local to a column: the owner of column k + 1 brings that column up to date first, searches the
+// pivot (integer images of the non-negative binary64 |.|^2, which order them exactly; the first row
+// on ties; a NaN never wins) while every row's thread divides 1 / |.|^2, and sends the column to the
+// CTAs with st.async (distributed shared memory, completing the bytes of a barrier per message)
+// before it turns to its other columns.  Messages go to a ring of GJC_SLOTS; a cluster barrier every
+// half ring keeps a slow reader's messages from being overwritten.
+// The binary64 pipe bounds the arithmetic: 4 w^3 multiply-adds at 2 a clock per SM are 253 us for
+// w = 64 on one SM, and one block of a launch has the whole GPU: the one-CTA forms (block in shared
+// memory: 423 us; in registers: 350 us) left 7/8 or more of it idle in single solves and small
+// batches.  C and the figures of each: launch_gjinv.
+// Same operations on every element as the one-CTA form of the block's order, so a block comes out the
+// same in a launch of any size up to one block per SM; `from_zero`: column k of the inverse by the
+// multiply-adds of the elimination applied to zero (gjinv_reg_kernel) instead of the negated product.
+constexpr int GJC_SLOTS = 32, GJC_MAX_C = 8;
+struct GjcHead { double2 pinv; int piv, sing, pad0, pad1; };
+
+__device__ __forceinline__ void st_async16(uint32_t addr, uint32_t bar, double2 v) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(addr),
+               "l"(__double_as_longlong(v.x)), "l"(__double_as_longlong(v.y)), "r"(bar) : "memory");
+}
+__device__ __forceinline__ uint32_t mapa_u32(uint32_t addr, int cta) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(cta));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(GJINV_THREADS)
+gjinv_cluster_kernel(const GjParams p, int C, int max_w) {
+  extern __shared__ double2 dyn[];          // [columns of this CTA][max_w], then the ring [GJC_SLOTS][max_w + 2]
+  __shared__ uint64_t bar[GJC_SLOTS];
+  __shared__ double2 xrow[GJINV_MAX / 2 + 1], okrow[GJINV_MAX / 2 + 1];   // new row k, old row k (own columns)
+  __shared__ long long wkey[GJINV_THREADS / 32];
+  __shared__ int wrow[GJINV_THREADS / 32];
+  __shared__ int dst[GJINV_MAX];            // column j of the block is column dst[j] of X
+  __shared__ int gave_up;
+  const int z = blockIdx.x / C, rank = blockIdx.x % C;
+  const bool single = p.D == nullptr;
+  const int w = single ? p.nb1 : p.nb[z];
+  if (w <= 0) return;                       // the same for the whole cluster
+  const bool from_zero = w > GJR_MIN_W && w <= GJR_W;
+  const double2* D = single ? p.D1 : p.D[z];
+  const long long ldd = single ? p.ldd1 : p.ldd[z];
+  double2* X = single ? p.X1 : p.X[z];
+  const long long ldx = single ? p.ldx1 : p.ldx[z];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int ncol = (w - rank + C - 1) / C;  // own columns (rank + C i < w); may be 0
+  double2* A = dyn;
+  double2* ring = dyn + static_cast<size_t>((max_w + C - 1) / C) * max_w;
+  const int pitch = max_w + 2;              // ring slot: the column, then the head
+  const uint32_t msg_bytes = static_cast<uint32_t>(w + 2) * sizeof(double2);
+  // row r of the columns cg, cg + ng, ... is this thread's
+  const int wp = w <= 64 ? 64 : 128, r = tid & (wp - 1), cg = tid / wp, ng = GJINV_THREADS / wp;
+  for (int jl = cg; jl < ncol; jl += ng)
+    if (r < w) A[jl * max_w + r] = D[r + (rank + static_cast<long long>(C) * jl) * ldd];
+  if (tid < w) dst[tid] = tid;
+  if (tid == 0) {
+    gave_up = 0;
+    for (int i = 0; i < GJC_SLOTS; ++i) mbar_init(&bar[i], 1);
+    mbar_fence_init();
+    for (int i = 0; i < GJC_SLOTS && i < w; ++i) mbar_arrive_expect_tx(&bar[i], msg_bytes);
+  }
+  __syncthreads();
+  cluster_sync();
+
+  // thread r < w holds v = entry r of column k (up to date): pivot search among rows >= k and the
+  // message of column k to every CTA (all threads of the CTA take part)
+  auto send = [&](int k, double2 v) {
+    long long key = -1;
+    double inv = 0.0;
+    if (tid < w) {
+      const double a2 = v.x * v.x + v.y * v.y;
+      if (tid >= k) key = __double_as_longlong(a2);
+      if (key > 0x7FF0000000000000LL) key = -1;             // NaN
+      inv = 1.0 / a2;                                       // the one division of the step, ahead of the choice
+    }
+    int bi = tid;
+    long long best = key;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+    }
+    if (lane == 0) { wkey[tid >> 5] = best; wrow[tid >> 5] = bi; }
+    __syncthreads();
+    best = wkey[0];
+    bi = wrow[0];
+    for (int q = 1; 32 * q < w; ++q)
+      if (wkey[q] > best) { best = wkey[q]; bi = wrow[q]; }
+    const bool sing = best <= 0;
+    if (sing) bi = k;
+    if (tid < w) {
+      const uint32_t slot = smem_u32(ring + static_cast<size_t>(k % GJC_SLOTS) * pitch);
+      const uint32_t b = smem_u32(&bar[k % GJC_SLOTS]);
+      // the exchange: row k's entry goes to the pivot's place, the pivot row's multiplier is zero
+      const int pos = tid == bi ? k : (tid == k ? bi : tid);
+      const double2 out = tid == bi ? make_double2(0.0, 0.0) : v;
+      for (int c = 0; c < C; ++c) {
+        const uint32_t rs = mapa_u32(slot, c), rb = mapa_u32(b, c);
+        st_async16(rs + static_cast<uint32_t>(pos * sizeof(double2)), rb, out);
+        if (tid == bi) {
+          const double2 head1 = make_double2(__hiloint2double(sing ? 1 : 0, bi), 0.0);
+          st_async16(rs + static_cast<uint32_t>(w * sizeof(double2)), rb, make_double2(v.x * inv, -v.y * inv));
+          st_async16(rs + static_cast<uint32_t>((w + 1) * sizeof(double2)), rb, head1);
+        }
+      }
+    }
+  };
+
+  if (rank == 0) send(0, r < w && cg == 0 ? A[r] : make_double2(0.0, 0.0));
+  bool singular = false;
+  for (int k = 0; k < w; ++k) {
+    if (k > 0 && k % (GJC_SLOTS / 2) == 0) cluster_sync();  // every CTA is done with the steps below k
+    if (gave_up) continue;                                  // (only the cluster's barriers are kept)
+    const int slot = k % GJC_SLOTS;
+    const double2* msg = ring + static_cast<size_t>(slot) * pitch;
+    {
+      const uint32_t parity = static_cast<uint32_t>(k / GJC_SLOTS) & 1u;
+      const long long t0 = clock64();
+      while (!mbar_try_wait(&bar[slot], parity))
+        if (clock64() - t0 > kWaitBudget) { gave_up = 1; break; }
+    }
+    __syncthreads();
+    if (gave_up) continue;
+    const double2 pinv = msg[w], head = msg[w + 1];
+    const int piv = __double2loint(head.x);
+    if (__double2hiint(head.x) != 0) { singular = true; break; }
+    if (tid == 0) {
+      if (k + GJC_SLOTS < w) mbar_arrive_expect_tx(&bar[slot], msg_bytes);
+      const int d = dst[k];
+      dst[k] = dst[piv];
+      dst[piv] = d;
+    }
+    const bool ahead = k + 1 < w && (k + 1) % C == rank;    // this CTA sends the next column
+    const int jn = (k + 1) / C;                             // its local index
+    if (ahead) {
+      double2 v = make_double2(0.0, 0.0);
+      double2* col = A + static_cast<size_t>(jn) * max_w;
+      if (tid < w) {
+        const double2 x = cmul(col[piv], pinv);
+        if (tid == k) {
+          v = x;
+        } else {
+          v = tid == piv ? col[k] : col[tid];
+          const double2 fr = msg[tid];
+          v.x = fma(-fr.x, x.x, v.x);
+          v.x = fma(fr.y, x.y, v.x);
+          v.y = fma(-fr.x, x.y, v.y);
+          v.y = fma(-fr.y, x.x, v.y);
+        }
+      }
+      __syncthreads();
+      if (tid < w) col[tid] = v;
+      send(k + 1, v);
+    }
+    if (tid < ncol) {
+      const double2* col = A + static_cast<size_t>(tid) * max_w;
+      xrow[tid] = cmul(col[piv], pinv);
+      okrow[tid] = col[k];
+    }
+    __syncthreads();
+    if (r < w) {
+      const double2 fr = msg[r];
+      for (int jl = cg; jl < ncol; jl += ng) {
+        if (ahead && jl == jn) continue;
+        double2* e = A + static_cast<size_t>(jl) * max_w + r;
+        if (rank + C * jl == k) {                           // column k of the inverse
+          double2 y;
+          if (from_zero) {
+            y.x = fma(-fr.x, pinv.x, 0.0);
+            y.x = fma(fr.y, pinv.y, y.x);
+            y.y = fma(-fr.x, pinv.y, 0.0);
+            y.y = fma(-fr.y, pinv.x, y.y);
+          } else {
+            const double2 c = cmul(fr, pinv);
+            y = make_double2(-c.x, -c.y);
+          }
+          *e = r == k ? pinv : y;
+          continue;
+        }
+        const double2 x = xrow[jl];
+        double2 y = r == piv ? okrow[jl] : *e;
+        y.x = fma(-fr.x, x.x, y.x);
+        y.x = fma(fr.y, x.y, y.x);
+        y.y = fma(-fr.x, x.y, y.y);
+        y.y = fma(-fr.y, x.x, y.y);
+        *e = r == k ? x : y;
+      }
+    }
+    __syncthreads();
+  }
+  if (tid == 0 && gave_up) flag_error(p.status, OZK_ERR_TIMEOUT);
+  if (singular && tid == 0 && rank == 0) flag_error(p.status, OZK_ERR_SINGULAR);
+  __syncthreads();
+  for (int jl = cg; jl < ncol; jl += ng)
+    if (r < w) X[r + static_cast<long long>(dst[rank + C * jl]) * ldx] =
+        singular ? make_double2(0.0, 0.0) : A[static_cast<size_t>(jl) * max_w + r];
+  // no CTA leaves while another may still send to it (every message is received before its step, but
+  // a singular or abandoned block ends early)
+  cluster_sync();
 }
 
 // In-place LU factorisation with partial pivoting of a w x w pivot block (w <= GJINV_MAX,
@@ -621,12 +829,39 @@ void launch_tri_inv(const double2* T, long long ldt, int r, int upper, int unit,
 }
 
 void launch_gjinv(const GjParams& p, int max_w, int batch, cudaStream_t st) {
-  // the register form takes the blocks of order 56 < w <= 64 when every block of the launch
-  // has an SM to itself, the shared-memory kernel the others; which form inverts a block
-  // depends on its own order and the launch's size only, so a block comes out the same alone
-  // and in a small batch
+  // A cluster per block while the launch leaves SMs idle: 8, 4 or 2 CTAs, as many as every block can
+  // have an SM for each.  64 x 64 blocks: 1 of them 135 us with 8 CTAs (350 in registers, 443 in
+  // shared memory by one CTA), 16 of them 190 us with 8 or 4, 38 of them 280 us with 2 or 4, 76 of
+  // them 280 us with 2; 152 of them 438 us with 2, so with more than an SM for every two blocks the
+  // one-CTA forms stay: the register form for blocks of order 56 < w <= 64 when every block of the
+  // launch has an SM to itself, the shared-memory kernel for the others.  Order 50: 106 us for one
+  // block with 8 CTAs against 275; order 112: 406 against 1831.  Which arithmetic inverts a block
+  // depends on its own order and on whether the launch has at most one block per SM only, so a block
+  // comes out the same alone and in a small batch.
+  const int sms = gpu_sm_count();
+  const int C = 8 * batch <= sms ? 8 : (4 * batch <= sms ? 4 : (2 * batch <= sms ? 2 : 1));
+  if (C > 1) {
+    const size_t smem = sizeof(double2) * (static_cast<size_t>((max_w + C - 1) / C) * max_w +
+                                           static_cast<size_t>(GJC_SLOTS) * (max_w + 2));
+    cudaFuncSetAttribute(gjinv_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(static_cast<unsigned>(batch * C));
+    cfg.blockDim = dim3(GJINV_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = static_cast<unsigned>(C);
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, gjinv_cluster_kernel, p, C, max_w);
+    record_launch();
+    return;
+  }
   const bool single = p.D == nullptr;                      // one block, of order max_w
-  const bool reg = max_w > GJR_MIN_W && batch <= gpu_sm_count() && (!single || max_w <= GJR_W);
+  const bool reg = max_w > GJR_MIN_W && batch <= sms && (!single || max_w <= GJR_W);
   if (reg) {
     gjinv_reg_kernel<<<batch, GJR_THREADS, 0, st>>>(p);
     record_launch();
