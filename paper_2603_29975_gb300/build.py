@@ -16,7 +16,8 @@ SRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libozk.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["split.cu", "slice_gemm.cu", "slice_gemm_s345.cu", "slice_gemm_s678.cu", "dmma.cu", "lu.cu", "selector.cu", "ozaki2.cu", "api.cu"]
+SOURCES = ["split.cu", "slice_gemm.cu", "slice_gemm_s345.cu", "slice_gemm_s678.cu",
+           "slice_gemm_s910.cu", "dmma.cu", "lu.cu", "selector.cu", "ozaki2.cu", "api.cu"]
 
 
 def nvcc() -> str:

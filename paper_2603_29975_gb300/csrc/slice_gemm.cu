@@ -1,6 +1,7 @@
 // Launchers of the slice-pair GEMM (kernel: slice_gemm.cuh) and its small helpers: the finishing
 // kernel of a split K and the tile prefix sums of a batch.  The run-time instances of the kernel are
-// compiled here, the compile-time slice counts in slice_gemm_s345.cu and slice_gemm_s678.cu.
+// compiled here, the compile-time slice counts in slice_gemm_s345.cu, slice_gemm_s678.cu and
+// slice_gemm_s910.cu.
 #include <algorithm>
 
 #include "slice_gemm.cuh"
@@ -44,12 +45,14 @@ void launch_slice_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const GemmP
   const int grid = static_cast<int>(std::min<long long>(ntiles, num_sms()));
   const size_t smem = gemm_smem_bytes(p.S, BN, p.nstage);
   // the compile-time instances hold only the fast epilogues (no integer group dumps)
-  const bool tri = BN == 64 && !p.fullset && !p.diag_pairs && p.mode != EPI_GROUPS && p.mode != EPI_RESIDUES;
+  const bool tri = !p.fullset && !p.diag_pairs && p.mode != EPI_GROUPS && p.mode != EPI_RESIDUES;
   const bool ks = p.ksplit > 1;
   // 23 to 63 bits (S = 3..8): compact instances of one schedule and epilogue each; split K only for
   // S = 7, the precision of the batched contour workload (its unit bookkeeping costs the others
   // registers)
-  if (tri && p.S >= 3 && p.S <= 8 && (!ks || p.S == 7)) {
+  if (tri && BN == 32 && (p.S == 9 || p.S == 10)) {
+    launch_slice_gemm_s910(ta, tb, p, grid, smem, st);
+  } else if (tri && BN == 64 && p.S >= 3 && p.S <= 8 && (!ks || p.S == 7)) {
     if (p.S <= 5) launch_slice_gemm_s345(ta, tb, p, grid, smem, st);
     else launch_slice_gemm_s678(ta, tb, p, grid, smem, st);
   } else if (BN == 64) {

@@ -624,6 +624,93 @@ __device__ __forceinline__ bool epilogue_fast(const GemmParams& p, const EpiCtx&
   return true;
 }
 
+// Epilogue of one 128 x 32 tile for G = 9 or 10 groups (S = 9, 10): as epilogue_fast with the groups
+// in quads, each folded into a 64-bit sum per stacked column (8 columns a thread), combined to the
+// 128-bit sum and rounded at the end of the tile.  Taken with a 128-bit shift and add and the
+// conversion unit per accumulator and chunk instead, the drains bound 2048^3 at S = 10: 6.0 ms.
+template <int G>
+struct WidePlan {
+  __host__ __device__ static constexpr int quad_end(int g) { return (g / 4) * 4 + 4 < G ? (g / 4) * 4 + 4 : G; }
+  __host__ __device__ static constexpr int ng(int g) { return quad_end(g) - g >= 2 ? 2 : 1; }
+  __host__ __device__ static constexpr int shift(int g) { return 8 * (quad_end(g) - g - ng(g)); }
+  __host__ __device__ static constexpr unsigned long long bias(int quad) {
+    unsigned long long b = 0;
+    for (int g = 4 * quad; g < G && g < 4 * quad + 4; g += ng(g))
+      b += static_cast<unsigned long long>(ng(g) == 2 ? MAGIC_PAIR : MAGIC_ONE) << shift(g);
+    return b;
+  }
+};
+template <int G, int GI, int GE, bool REDO>
+__device__ __forceinline__ void wide_steps(uint32_t tbase, uint64_t* acc_empty, int lane, bool early, float& big,
+                                           unsigned long long (&X)[3][8]) {
+  using P = WidePlan<G>;
+  if constexpr (GI < GE) {
+    constexpr int BN = 32, ng = P::ng(GI);
+    uint32_t v[8], u[8];
+    tmem_ld8(tbase + GI * BN, v);
+    if constexpr (ng == 2) tmem_ld8(tbase + (GI + 1) * BN, u);
+    tmem_wait_ld();
+    if constexpr (REDO) {
+      if constexpr (ng == 2) refold_pair<P::shift(GI)>(X[GI / 4], v, u);
+      else refold_one<P::shift(GI)>(X[GI / 4], v);
+    } else {
+      if (early) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          mbar_arrive(&acc_empty[GI]);
+          if constexpr (ng == 2) mbar_arrive(&acc_empty[GI + 1]);
+        }
+      }
+      big = max_abs(big, v);
+      if constexpr (ng == 2) big = max_abs(big, u);
+      if constexpr (ng == 2) fold_pair<P::shift(GI)>(X[GI / 4], v, u);
+      else fold_one<P::shift(GI)>(X[GI / 4], v);
+    }
+    wide_steps<G, GI + ng, GE, REDO>(tbase, acc_empty, lane, early, big, X);
+  }
+}
+template <int G, int G0, int GE>
+__device__ __forceinline__ bool wide_part(uint32_t tbase, uint64_t* acc_empty, int lane, uint32_t magic_mask,
+                                          ChunkWait& cw, unsigned long long (&X)[3][8]) {
+  if (!cw.part(G0 == 0 ? 0 : 1)) return false;
+  constexpr uint32_t need = ((1u << (GE - G0)) - 1u) << G0;
+  const bool known = (magic_mask & need) == need;
+  float big = 0.0f;
+  wide_steps<G, G0, GE, false>(tbase, acc_empty, lane, known, big, X);
+  if (!known) {
+    if (__any_sync(0xffffffffu, !(big < 4194304.0f))) wide_steps<G, G0, GE, true>(tbase, acc_empty, lane, false, big, X);
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) {
+#pragma unroll
+      for (int g = G0; g < GE; ++g) mbar_arrive(&acc_empty[g]);
+    }
+  }
+  return true;
+}
+// the exact sums T of the thread's 8 columns over the tile's chunks
+template <int G>
+__device__ __forceinline__ bool wide_sums(uint32_t tbase, uint64_t* acc_empty, int lane, uint32_t magic_mask, ChunkWait& cw,
+                                          __int128 (&T)[8]) {
+  unsigned long long X[3][8];
+#pragma unroll
+  for (int q = 0; q < 3; ++q)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) X[q][j] = 0ull - static_cast<unsigned long long>(cw.nchunks) * WidePlan<G>::bias(q);
+  for (int c = 0; c < cw.nchunks; ++c) {
+    if (!wide_part<G, 0, split_group(G)>(tbase, acc_empty, lane, magic_mask, cw, X)) return false;
+    if (!wide_part<G, split_group(G), G>(tbase, acc_empty, lane, magic_mask, cw, X)) return false;
+    ++*cw.cc;
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    T[j] = (static_cast<__int128>(static_cast<long long>(X[0][j])) << (8 * (G - 4))) +
+           (static_cast<__int128>(static_cast<long long>(X[1][j])) << (8 * (G - 8))) +
+           static_cast<__int128>(static_cast<long long>(X[2][j]));
+  return true;
+}
+
 // SF = 0: the slice count, pair schedule and epilogue variant are chosen at run time.  SF > 0:
 // an instance for S = SF with the triangular pair set only, whose MMA issuer and epilogue
 // contain just that schedule and group count -- the tensor pipe is fed markedly faster from
@@ -994,14 +1081,18 @@ slice_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           continue;
         }
       }
-      if constexpr (SF == 0) {                   // compile-time instances take only the fast epilogues
+      if constexpr (SF == 0 || BN == 32) {       // 64-column compile-time instances take only the fast epilogues
         const bool horner = unch == 1;
         const int row = ti->row0 + rl, n0 = ti->n0, n2_z = ti->n2, z = ti->z;
         const bool rowok = rl < ti->rows;
         __int128 T[COLS];
 #pragma unroll
         for (int j = 0; j < COLS; ++j) T[j] = 0;
-        for (int c = 0; c < unch; ++c, ++cc) {
+        if constexpr (SF > 0 && BN == 32) {
+          ChunkWait cw{acc_full, unch, &cc, p.status, abort_flag};
+          if (!wide_sums<SF>(tbase, acc_empty, lane, magic_mask, cw, T)) ok = false;
+        }
+        for (int c = 0; SF == 0 && c < unch; ++c, ++cc) {
           // (every group after the second part: these forms are not bound by the boundary)
           if (!mbar_wait(&acc_full[0], cc & 1, p.status, abort_flag) ||
               !mbar_wait(&acc_full[1], cc & 1, p.status, abort_flag)) { ok = false; break; }
@@ -1086,8 +1177,11 @@ inline void launch_instance(const CUtensorMap& ta, const CUtensorMap& tb, const 
                        static_cast<int>(smem));
   slice_gemm_kernel<BN, SF, KS><<<grid, GEMM_THREADS, smem, st>>>(ta, tb, p);
 }
-// the instances of S = 3..5 and of S = 6..8 (split K: S = 7), each in its own translation unit
+// the instances of S = 3..5, of S = 6..8 (split K: S = 7) and of S = 9, 10, each in its own
+// translation unit
 void launch_slice_gemm_s345(const CUtensorMap& ta, const CUtensorMap& tb, const GemmParams& p, int grid, size_t smem,
+                            cudaStream_t st);
+void launch_slice_gemm_s910(const CUtensorMap& ta, const CUtensorMap& tb, const GemmParams& p, int grid, size_t smem,
                             cudaStream_t st);
 void launch_slice_gemm_s678(const CUtensorMap& ta, const CUtensorMap& tb, const GemmParams& p, int grid, size_t smem,
                             cudaStream_t st);
