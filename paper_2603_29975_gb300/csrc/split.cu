@@ -26,8 +26,8 @@ constexpr int SPLIT_ROWS = 32;               // rows of a CTA: one per lane
 constexpr int SPLIT_MAX_WARPS = 8;           // a warp takes one K-block (8 elements) at a time
 constexpr int SPLIT_MAX_KG = 8;              // CTAs of a cluster that share a row block's K-blocks
 
-// Digits of 8 elements for a compile-time slice count SF <= 8 (nbits = 8 SF - 1, 64-bit images),
-// with no dependent chain per digit.  With C = 128 (1 + 256 + ... + 256^(SF-2)), Y = X + C holds
+// Digits of 8 elements for a compile-time slice count SF <= 10 (nbits = 8 SF - 1; 64-bit images, 96-bit
+// ones for SF = 9 and 10), with no dependent chain per digit.  With C = 128 (1 + 256 + ... + 256^(SF-2)), Y = X + C holds
 // the balanced digits d_s + 128 of the SF - 1 lower places as its low bytes and the top digit
 // as Y >> 8 (SF - 1): X = sum_s d_s 256^s with every lower d_s in [-128, 127], so adding 128
 // at each lower place lifts it into [0, 255] without carries, and base-256 digits are unique.
@@ -111,13 +111,13 @@ __device__ __forceinline__ void store_slice(const SplitDst<SIDE>& d, int s, cons
   }
 }
 
-// The integer image X = trunc(x 2^(nbits - e)) of |x| < 2^e, nbits =
+// The integer image X = trunc(x 2^(nbits - e)) of |x| < 2^e, e >= -1021, nbits =
 // 8 SF - 1: the 53-bit significand, shifted left by the constant max(0, nbits - 53) that no element
 // exceeds, then right.  (Rows flagged non-finite have e = 0, which does not bound their finite
 // elements: those are cut to the significand's range.)
 template <int SF>
 __device__ __forceinline__ long long image_fixed(long long bits, int e) {
-  constexpr int nbits = 8 * SF - 1, left = nbits > 53 ? nbits - 53 : 0;
+  constexpr int nbits = 8 * SF - 1, left = nbits > 53 ? (nbits - 53) % 64 : 0;
   const int ex = static_cast<int>(bits >> 52) & 0x7FF;
   const unsigned long long man = static_cast<unsigned long long>(bits) & ((1ull << 52) - 1ull);
   const unsigned long long M = ex == 0 ? man : (man | (1ull << 52));
@@ -126,13 +126,44 @@ __device__ __forceinline__ long long image_fixed(long long bits, int e) {
   return bits < 0 ? -mag : mag;
 }
 
+// the same for SF = 9, 10 plus the bias: Y = C + X in three words (the significand shifted left by up
+// to 18 or 26 bits)
+template <int SF>
+__device__ __forceinline__ void image_wide(long long bits, int e, uint32_t& w0, uint32_t& w1, uint32_t& w2) {
+  constexpr int nbits = 8 * SF - 1, left = nbits - 53;
+  const int ex = static_cast<int>(bits >> 52) & 0x7FF;
+  const unsigned long long man = static_cast<unsigned long long>(bits) & ((1ull << 52) - 1ull);
+  const unsigned long long M = ex == 0 ? man : (man | (1ull << 52));
+  const int right = max(e + (left + 1075 - nbits) - max(ex, 1), 0);
+  const int up = max(left - right, 0);
+  unsigned long long lo = (M << up) >> min(max(right - left, 0), 63);
+  uint32_t hi = up > 11 ? static_cast<uint32_t>(M >> (64 - up)) : 0u;
+  if (bits < 0) {
+    hi = ~hi + (lo == 0ull ? 1u : 0u);
+    lo = 0ull - lo;
+  }
+  constexpr unsigned long long Clo = 0x8080808080808080ull;             // bytes 0..7
+  constexpr uint32_t Chi = SF == 9 ? 0u : 0x80u;                         // byte 8 (SF = 10)
+  const unsigned long long s = lo + Clo;
+  hi += Chi + (s < lo ? 1u : 0u);
+  w0 = static_cast<uint32_t>(s);
+  w1 = static_cast<uint32_t>(s >> 32);
+  w2 = hi;
+}
+
 template <int SF, int SIDE>
 __device__ __forceinline__ void emit_fixed(const SplitDst<SIDE>& d, const longlong2 (&v)[8], int e) {
-  constexpr long long C = digit_bias(SF);
+  constexpr long long C = SF <= 8 ? digit_bias(SF <= 8 ? SF : 8) : 0;
   uint32_t rl[8], rh[8], il[8], ih[8];                    // low and high words of Y
   uint32_t tr[4], ti[4];                                  // SF = 8: the top digits, two a word
+  uint32_t rx[8], ix[8];                                  // SF > 8: third words
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
+    if constexpr (SF > 8) {
+      image_wide<SF>(v[q].x, e, rl[q], rh[q], rx[q]);
+      image_wide<SF>(v[q].y, e, il[q], ih[q], ix[q]);
+      continue;
+    }
     const long long xr = image_fixed<SF>(v[q].x, e), xi = image_fixed<SF>(v[q].y, e);
     const unsigned long long a = static_cast<unsigned long long>(xr) + C, b = static_cast<unsigned long long>(xi) + C;
     rl[q] = static_cast<uint32_t>(a); rh[q] = static_cast<uint32_t>(a >> 32);
@@ -153,13 +184,21 @@ __device__ __forceinline__ void emit_fixed(const SplitDst<SIDE>& d, const longlo
       uint32_t br, bi;
       if (s > 0) {
         const uint32_t sel = static_cast<uint32_t>(k & 3) | (static_cast<uint32_t>((k & 3) + 4) << 8);
-        br = (__byte_perm(k < 4 ? rl[2 * h] : rh[2 * h], k < 4 ? rl[2 * h + 1] : rh[2 * h + 1], sel) & 0x00FF00FFu) +
+        br = (__byte_perm(k < 4 ? rl[2 * h] : (k < 8 ? rh[2 * h] : rx[2 * h]),
+                          k < 4 ? rl[2 * h + 1] : (k < 8 ? rh[2 * h + 1] : rx[2 * h + 1]), sel) & 0x00FF00FFu) +
              0x65806580u;
-        bi = (__byte_perm(k < 4 ? il[2 * h] : ih[2 * h], k < 4 ? il[2 * h + 1] : ih[2 * h + 1], sel) & 0x00FF00FFu) +
+        bi = (__byte_perm(k < 4 ? il[2 * h] : (k < 8 ? ih[2 * h] : ix[2 * h]),
+                          k < 4 ? il[2 * h + 1] : (k < 8 ? ih[2 * h + 1] : ix[2 * h + 1]), sel) & 0x00FF00FFu) +
              0x65806580u;
       } else if constexpr (SF == 8) {
         br = tr[h];
         bi = ti[h];
+      } else if constexpr (SF > 8) {                        // the top digit: third word from byte SF - 9 on
+        constexpr int sh = 8 * (SF - 9);
+        br = __byte_perm(static_cast<uint32_t>((static_cast<int>(rx[2 * h]) >> sh) + 0x6600),
+                         static_cast<uint32_t>((static_cast<int>(rx[2 * h + 1]) >> sh) + 0x6600), 0x5410);
+        bi = __byte_perm(static_cast<uint32_t>((static_cast<int>(ix[2 * h]) >> sh) + 0x6600),
+                         static_cast<uint32_t>((static_cast<int>(ix[2 * h + 1]) >> sh) + 0x6600), 0x5410);
       } else {
         br = top_pair<SF>(rl[2 * h], rh[2 * h], rl[2 * h + 1], rh[2 * h + 1]);
         bi = top_pair<SF>(il[2 * h], ih[2 * h], il[2 * h + 1], ih[2 * h + 1]);
@@ -326,10 +365,21 @@ __device__ __forceinline__ void split_rows(const SplitParams& p, unsigned long l
         if (abs_bits(v[q].y) >= 0x7FF0000000000000ull) v[q].y = 0;
       }
     }
+    // rows of subnormal numbers: their significands are shorter than their exponent says, so they are
+    // scaled (exactly) into the normal range, and the exponent with them
+    int ei = e;
+    if (SF > 0 && e < -1000) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        v[q].x = __double_as_longlong(__longlong_as_double(v[q].x) * 0x1.0p100);
+        v[q].y = __double_as_longlong(__longlong_as_double(v[q].y) * 0x1.0p100);
+      }
+      ei += 100;
+    }
     d.out = outz + 2LL * kb * d.hplane + (SIDE == 0 ? r : 2 * r);
     d.tail4 = K - 8 * kb <= 4;
     d.has2 = 2 * kb + 1 < halves;
-    if constexpr (SF > 0) emit_fixed<SF, SIDE>(d, v, e);
+    if constexpr (SF > 0) emit_fixed<SF, SIDE>(d, v, ei);
     else emit_generic<W64, SIDE>(p, d, v, e, r, 8 * kb, K, z == 0 ? p.dbg_digits : nullptr);
   }
 }
@@ -372,7 +422,7 @@ void launch_split(const SplitParams& a, int rows_a, const SplitParams* b, int ro
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = kg > 1 ? 1 : 0;
-  // compile-time slice counts 3..8 (nbits = 8 S - 1 on every side); the test hook's digit copy and
+  // compile-time slice counts 3..10 (nbits = 8 S - 1 on every side); the test hook's digit copy and
   // other slice counts take the run-time form
   int sf = pp.s[0].S;
   for (int sd = 0; sd < pp.nsides; ++sd)
@@ -384,6 +434,8 @@ void launch_split(const SplitParams& a, int rows_a, const SplitParams* b, int ro
     case 6: cudaLaunchKernelEx(&cfg, split_kernel<6, true>, pp); break;
     case 7: cudaLaunchKernelEx(&cfg, split_kernel<7, true>, pp); break;
     case 8: cudaLaunchKernelEx(&cfg, split_kernel<8, true>, pp); break;
+    case 9: cudaLaunchKernelEx(&cfg, split_kernel<9, false>, pp); break;
+    case 10: cudaLaunchKernelEx(&cfg, split_kernel<10, false>, pp); break;
     default:
       if (pp.s[0].nbits <= 62 && (pp.nsides < 2 || pp.s[1].nbits <= 62)) cudaLaunchKernelEx(&cfg, split_kernel<0, true>, pp);
       else cudaLaunchKernelEx(&cfg, split_kernel<0, false>, pp);

@@ -50,12 +50,14 @@ def test_accumulators_beyond_the_small_range(ozk_mod, handle, S, k):
     assert np.array_equal(_product(ozk_mod, handle, A, B, S), co.zgemm(A, B, S))
 
 
-@pytest.mark.parametrize("S", [4, 7])
-@pytest.mark.parametrize("pa,pb", [(-500, -480), (-540, -530), (500, 480), (600, -560), (520, 503)])
+@pytest.mark.parametrize("S", [3, 4, 7, 8, 10])
+@pytest.mark.parametrize("pa,pb", [(-500, -480), (-540, -530), (500, 480), (600, -560), (520, 503), (-1030, 900),
+                                   (-1060, 1000), (980, -1050)])
 def test_exponents_at_the_ends_of_the_range(ozk_mod, handle, S, pa, pb):
-    A, B = rand_complex(37, 20, seed=9) * 2.0 ** pa, rand_complex(20, 35, seed=10) * 2.0 ** pb
-    A[3] *= 2.0 ** (-pa)                                  # ordinary rows and columns in the same tile
-    B[:, 5] *= 2.0 ** (-pb)
+    A, B = rand_complex(37, 20, seed=9), rand_complex(20, 35, seed=10)
+    # all but one row and one column (ordinary ones in the same tile)
+    A[np.arange(37) != 3] *= 2.0 ** pa
+    B[:, np.arange(35) != 5] *= 2.0 ** pb
     assert np.array_equal(_product(ozk_mod, handle, A, B, S), co.zgemm(A, B, S))
 
 
