@@ -463,27 +463,32 @@ gjinv_reg_kernel(const GjParams p) {
 }
 
 // The same Gauss-Jordan inversion with each block spread over a cluster of C CTAs (2, 4 or 8): CTA c
-// keeps the columns c, c + C, ... of its block in shared memory.  A step needs column k (after the
-// exchange, its multipliers), the pivot's row and its reciprocal in every CTA, everything else is
-// local to a column: the owner of column k + 1 brings that column up to date first, searches the
-// pivot (integer images of the non-negative binary64 |.|^2, which order them exactly; the first row
-// on ties; a NaN never wins) while every row's thread divides 1 / |.|^2, and sends the column to the
-// CTAs with st.async (distributed shared memory, completing the bytes of a barrier per message)
-// before it turns to its other columns.  Messages go to a ring of GJC_SLOTS; a cluster barrier every
-// half ring keeps a slow reader's messages from being overwritten.
+// keeps a run of nc = ceil(w / C) columns of its block in shared memory.  A step needs column k (after
+// the exchange, its multipliers), the pivot's row and its reciprocal in every CTA, everything else is
+// local to a column.  The steps are a serial chain -- bring column k + 1 up to date, search its pivot,
+// divide -- and nc of them in a row stay within one CTA: there the first warps (a thread per row, the
+// chain) do nothing else and leave the step's message in the CTA's own ring, while the other warps send
+// the message before it to the other CTAs (a bulk copy to each one's shared memory, completing the bytes
+// of a barrier per message) and bring the remaining columns up to date.  The pivot search orders integer
+// images of the non-negative binary64 |.|^2 (their order exactly; the first row on ties; a NaN never
+// wins) while every row's thread divides 1 / |.|^2.  Messages go to a ring of GJC_SLOTS; a cluster
+// barrier every half ring keeps a slow reader's messages from being overwritten.
 // The binary64 pipe bounds the arithmetic: 4 w^3 multiply-adds at 2 a clock per SM are 253 us for
-// w = 64 on one SM, and one block of a launch has the whole GPU: the one-CTA forms (block in shared
+// w = 64 on one SM (a scheduler takes one such instruction of a warp in 64 clocks, whatever its active
+// lanes, and gives the result as late: the chain's 17 a step are 1100 of the 2900 clocks that a step
+// takes, column k + 1, |.|^2 and the division one after the other), and one block of a launch has the whole GPU: the one-CTA forms (block in shared
 // memory: 423 us; in registers: 350 us) left 7/8 or more of it idle in single solves and small
-// batches.  C and the figures of each: launch_gjinv.
+// batches.  With the columns dealt round robin, so that every step's message crossed between CTAs on
+// the chain, and sent as 16-byte stores (st.async: about 8 clocks each, 528 a step), 8 CTAs took 135 us.  C and the figures of each: launch_gjinv.
 // Same operations on every element as the one-CTA form of the block's order, so a block comes out the
 // same in a launch of any size up to one block per SM; `from_zero`: column k of the inverse by the
 // multiply-adds of the elimination applied to zero (gjinv_reg_kernel) instead of the negated product.
-constexpr int GJC_SLOTS = 32, GJC_MAX_C = 8;
-struct GjcHead { double2 pinv; int piv, sing, pad0, pad1; };
+constexpr int GJC_SLOTS = 32, GJC_THREADS = 512;
 
-__device__ __forceinline__ void st_async16(uint32_t addr, uint32_t bar, double2 v) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(addr),
-               "l"(__double_as_longlong(v.x)), "l"(__double_as_longlong(v.y)), "r"(bar) : "memory");
+// shared memory of this CTA to another's, completing `bytes` of that CTA's barrier; 16-byte aligned
+__device__ __forceinline__ void bulk_to_cta(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "r"(src), "r"(bytes), "r"(bar) : "memory");
 }
 __device__ __forceinline__ uint32_t mapa_u32(uint32_t addr, int cta) {
   uint32_t r;
@@ -494,15 +499,20 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-__global__ void __launch_bounds__(GJINV_THREADS)
+// barrier of the first `n` threads (id 1) or of the others (id 2); n is a multiple of 32
+__device__ __forceinline__ void named_sync(int id, int n) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+
+__global__ void __launch_bounds__(GJC_THREADS)
 gjinv_cluster_kernel(const GjParams p, int C, int max_w) {
   extern __shared__ double2 dyn[];          // [columns of this CTA][max_w], then the ring [GJC_SLOTS][max_w + 2]
   __shared__ uint64_t bar[GJC_SLOTS];
   __shared__ double2 xrow[GJINV_MAX / 2 + 1], okrow[GJINV_MAX / 2 + 1];   // new row k, old row k (own columns)
-  __shared__ long long wkey[GJINV_THREADS / 32];
-  __shared__ int wrow[GJINV_THREADS / 32];
+  __shared__ unsigned long long wkey[4];
+  __shared__ int wrow[4];
   __shared__ int dst[GJINV_MAX];            // column j of the block is column dst[j] of X
-  __shared__ int gave_up;
+  __shared__ int gave_up;                   // 1 + the first step whose message did not come
   const int z = blockIdx.x / C, rank = blockIdx.x % C;
   const bool single = p.D == nullptr;
   const int w = single ? p.nb1 : p.nb[z];
@@ -513,97 +523,100 @@ gjinv_cluster_kernel(const GjParams p, int C, int max_w) {
   double2* X = single ? p.X1 : p.X[z];
   const long long ldx = single ? p.ldx1 : p.ldx[z];
   const int tid = threadIdx.x, lane = tid & 31;
-  const int ncol = (w - rank + C - 1) / C;  // own columns (rank + C i < w); may be 0
+  const int nc = (w + C - 1) / C, c0 = rank * nc;
+  const int ncol = max(0, min(nc, w - c0)); // own columns c0 + jl; the last CTAs may have none
   double2* A = dyn;
   double2* ring = dyn + static_cast<size_t>((max_w + C - 1) / C) * max_w;
   const int pitch = max_w + 2;              // ring slot: the column, then the head
   const uint32_t msg_bytes = static_cast<uint32_t>(w + 2) * sizeof(double2);
-  // row r of the columns cg, cg + ng, ... is this thread's
-  const int wp = w <= 64 ? 64 : 128, r = tid & (wp - 1), cg = tid / wp, ng = GJINV_THREADS / wp;
+  // row r of the columns cg, cg + ng, ... is this thread's; the chain is the first wp threads
+  const int wp = w <= 64 ? 64 : 128, r = tid & (wp - 1), cg = tid / wp, ng = GJC_THREADS / wp;
   for (int jl = cg; jl < ncol; jl += ng)
-    if (r < w) A[jl * max_w + r] = D[r + (rank + static_cast<long long>(C) * jl) * ldd];
+    if (r < w) A[jl * max_w + r] = D[r + (c0 + jl) * ldd];
   if (tid < w) dst[tid] = tid;
-  if (tid == 0) {
+  // the barrier of step k's slot completes with the message's bytes, or at once where this CTA writes
+  // the message itself
+  auto arm = [&](int k) {
+    if (k / nc == rank) mbar_arrive(&bar[k % GJC_SLOTS]);
+    else mbar_arrive_expect_tx(&bar[k % GJC_SLOTS], msg_bytes);
+  };
+  if (tid == GJC_THREADS - 1) {
     gave_up = 0;
     for (int i = 0; i < GJC_SLOTS; ++i) mbar_init(&bar[i], 1);
     mbar_fence_init();
-    for (int i = 0; i < GJC_SLOTS && i < w; ++i) mbar_arrive_expect_tx(&bar[i], msg_bytes);
+    for (int i = 0; i < GJC_SLOTS && i < w; ++i) arm(i);
   }
   __syncthreads();
   cluster_sync();
 
-  // thread r < w holds v = entry r of column k (up to date): pivot search among rows >= k and the
-  // message of column k to every CTA (all threads of the CTA take part)
-  auto send = [&](int k, double2 v) {
-    long long key = -1;
+  // the chain's thread r < w holds v = entry r of column k (up to date): pivot search among rows >= k,
+  // column k back into col and its message into this CTA's ring
+  auto search = [&](int k, double2 v, double2* col) {
+    unsigned long long key = 0;                             // 0: not a candidate, or |.|^2 = 0
     double inv = 0.0;
     if (tid < w) {
       const double a2 = v.x * v.x + v.y * v.y;
-      if (tid >= k) key = __double_as_longlong(a2);
-      if (key > 0x7FF0000000000000LL) key = -1;             // NaN
+      if (tid >= k) key = static_cast<unsigned long long>(__double_as_longlong(a2));
+      if (key > 0x7FF0000000000000ull) key = 0;             // NaN
       inv = 1.0 / a2;                                       // the one division of the step, ahead of the choice
     }
-    int bi = tid;
-    long long best = key;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-    }
+    const unsigned hi = static_cast<unsigned>(key >> 32), bh = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned lo = hi == bh ? static_cast<unsigned>(key) : 0u, bl = __reduce_max_sync(0xffffffffu, lo);
+    int bi = static_cast<int>(__reduce_min_sync(0xffffffffu, hi == bh && lo == bl ? static_cast<unsigned>(tid) : 1024u));
+    unsigned long long best = static_cast<unsigned long long>(bh) << 32 | bl;
     if (lane == 0) { wkey[tid >> 5] = best; wrow[tid >> 5] = bi; }
-    __syncthreads();
+    named_sync(1, wp);                                      // also: every read of col is done
     best = wkey[0];
     bi = wrow[0];
     for (int q = 1; 32 * q < w; ++q)
       if (wkey[q] > best) { best = wkey[q]; bi = wrow[q]; }
-    const bool sing = best <= 0;
+    const bool sing = best == 0;
     if (sing) bi = k;
     if (tid < w) {
-      const uint32_t slot = smem_u32(ring + static_cast<size_t>(k % GJC_SLOTS) * pitch);
-      const uint32_t b = smem_u32(&bar[k % GJC_SLOTS]);
+      double2* m = ring + static_cast<size_t>(k % GJC_SLOTS) * pitch;
       // the exchange: row k's entry goes to the pivot's place, the pivot row's multiplier is zero
-      const int pos = tid == bi ? k : (tid == k ? bi : tid);
-      const double2 out = tid == bi ? make_double2(0.0, 0.0) : v;
-      for (int c = 0; c < C; ++c) {
-        const uint32_t rs = mapa_u32(slot, c), rb = mapa_u32(b, c);
-        st_async16(rs + static_cast<uint32_t>(pos * sizeof(double2)), rb, out);
-        if (tid == bi) {
-          const double2 head1 = make_double2(__hiloint2double(sing ? 1 : 0, bi), 0.0);
-          st_async16(rs + static_cast<uint32_t>(w * sizeof(double2)), rb, make_double2(v.x * inv, -v.y * inv));
-          st_async16(rs + static_cast<uint32_t>((w + 1) * sizeof(double2)), rb, head1);
-        }
+      m[tid == bi ? k : (tid == k ? bi : tid)] = tid == bi ? make_double2(0.0, 0.0) : v;
+      if (tid == bi) {
+        m[w] = make_double2(v.x * inv, -v.y * inv);
+        m[w + 1] = make_double2(__hiloint2double(sing ? 1 : 0, bi), 0.0);
       }
+      col[tid] = v;
     }
   };
 
-  if (rank == 0) send(0, r < w && cg == 0 ? A[r] : make_double2(0.0, 0.0));
-  bool singular = false;
+  if (rank == 0 && tid < wp) search(0, tid < w ? A[tid] : make_double2(0.0, 0.0), A);
+  bool singular = false, quit = false;
   for (int k = 0; k < w; ++k) {
     if (k > 0 && k % (GJC_SLOTS / 2) == 0) cluster_sync();  // every CTA is done with the steps below k
-    if (gave_up) continue;                                  // (only the cluster's barriers are kept)
+    if (quit) continue;                                     // (only the cluster's barriers are kept)
     const int slot = k % GJC_SLOTS;
     const double2* msg = ring + static_cast<size_t>(slot) * pitch;
-    {
+    const bool mine = static_cast<unsigned>(k - c0) < static_cast<unsigned>(ncol);
+    if (!mine) {
       const uint32_t parity = static_cast<uint32_t>(k / GJC_SLOTS) & 1u;
       const long long t0 = clock64();
       while (!mbar_try_wait(&bar[slot], parity))
-        if (clock64() - t0 > kWaitBudget) { gave_up = 1; break; }
+        if (clock64() - t0 > kWaitBudget) { *static_cast<volatile int*>(&gave_up) = k + 1; break; }
     }
-    __syncthreads();
-    if (gave_up) continue;
+    __syncthreads();                                        // message k is here, the updates of step k - 1 are done
+    // a step's failed wait is seen by every thread after that step's barrier
+    if (!mine && *static_cast<volatile int*>(&gave_up) == k + 1) { quit = true; continue; }
+    // the chain goes on in this CTA
+    const bool ahead = static_cast<unsigned>(k + 1 - c0) < static_cast<unsigned>(ncol);
+    const int jn = k + 1 - c0;                              // its column's local index
+    const bool chain = ahead && tid < wp;
     const double2 pinv = msg[w], head = msg[w + 1];
     const int piv = __double2loint(head.x);
-    if (__double2hiint(head.x) != 0) { singular = true; break; }
-    if (tid == 0) {
-      if (k + GJC_SLOTS < w) mbar_arrive_expect_tx(&bar[slot], msg_bytes);
-      const int d = dst[k];
-      dst[k] = dst[piv];
-      dst[piv] = d;
+    const bool sing = __double2hiint(head.x) != 0;
+    if (mine && !chain && lane == 0) {                      // the others' copies of the message
+      const int c = (tid >> 5) - (ahead ? wp / 32 : 0);     // a warp a CTA
+      if (c < C && c != rank) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the message was written by plain stores
+        bulk_to_cta(mapa_u32(smem_u32(msg), c), smem_u32(msg), msg_bytes, mapa_u32(smem_u32(&bar[slot]), c));
+      }
     }
-    const bool ahead = k + 1 < w && (k + 1) % C == rank;    // this CTA sends the next column
-    const int jn = (k + 1) / C;                             // its local index
-    if (ahead) {
+    if (sing) { singular = true; break; }
+    if (chain) {
       double2 v = make_double2(0.0, 0.0);
       double2* col = A + static_cast<size_t>(jn) * max_w;
       if (tid < w) {
@@ -619,37 +632,43 @@ gjinv_cluster_kernel(const GjParams p, int C, int max_w) {
           v.y = fma(-fr.y, x.x, v.y);
         }
       }
-      __syncthreads();
-      if (tid < w) col[tid] = v;
-      send(k + 1, v);
+      search(k + 1, v, col);
+      continue;
     }
-    if (tid < ncol) {
-      const double2* col = A + static_cast<size_t>(tid) * max_w;
-      xrow[tid] = cmul(col[piv], pinv);
-      okrow[tid] = col[k];
+    if (tid == GJC_THREADS - 1) {
+      if (k + GJC_SLOTS < w) arm(k + GJC_SLOTS);
+      const int d = dst[k];
+      dst[k] = dst[piv];
+      dst[piv] = d;
     }
-    __syncthreads();
+    const int skip = ahead ? wp : 0;                        // the threads of the chain
+    if (tid >= skip && tid - skip < ncol && !(ahead && tid - skip == jn)) {
+      const double2* col = A + static_cast<size_t>(tid - skip) * max_w;
+      xrow[tid - skip] = cmul(col[piv], pinv);
+      okrow[tid - skip] = col[k];
+    }
+    if (ahead) named_sync(2, GJC_THREADS - wp);
+    else __syncthreads();
     if (r < w) {
       const double2 fr = msg[r];
-      for (int jl = cg; jl < ncol; jl += ng) {
-        if (ahead && jl == jn) continue;
+      // beside the chain its groups take all columns but column k + 1
+      const int q0 = ahead ? cg - 1 : cg, nq = ahead ? ng - 1 : ng, nt = ahead ? ncol - 1 : ncol;
+      for (int q = q0; q < nt; q += nq) {
+        const int jl = ahead && q >= jn ? q + 1 : q;
         double2* e = A + static_cast<size_t>(jl) * max_w + r;
-        if (rank + C * jl == k) {                           // column k of the inverse
-          double2 y;
-          if (from_zero) {
-            y.x = fma(-fr.x, pinv.x, 0.0);
-            y.x = fma(fr.y, pinv.y, y.x);
-            y.y = fma(-fr.x, pinv.y, 0.0);
-            y.y = fma(-fr.y, pinv.x, y.y);
-          } else {
-            const double2 c = cmul(fr, pinv);
-            y = make_double2(-c.x, -c.y);
-          }
-          *e = r == k ? pinv : y;
+        const bool inv_col = c0 + jl == k;                  // column k of the inverse: the same from zero, by pinv
+        if (inv_col && !from_zero) {
+          // the multiplier read again, volatile: else the compiler multiplies for every column and selects,
+          // and 4 of 8 operations of the bounding pipe are for nothing
+          const volatile double* fv = reinterpret_cast<const volatile double*>(msg + r);
+          const double fx = fv[0], fy = fv[1];
+          const double2 c = cmul(make_double2(fx, fy), pinv);
+          *e = r == k ? pinv : make_double2(-c.x, -c.y);
           continue;
         }
-        const double2 x = xrow[jl];
+        const double2 x = inv_col ? pinv : xrow[jl];
         double2 y = r == piv ? okrow[jl] : *e;
+        if (inv_col) y = make_double2(0.0, 0.0);
         y.x = fma(-fr.x, x.x, y.x);
         y.x = fma(fr.y, x.y, y.x);
         y.y = fma(-fr.x, x.y, y.y);
@@ -657,13 +676,12 @@ gjinv_cluster_kernel(const GjParams p, int C, int max_w) {
         *e = r == k ? x : y;
       }
     }
-    __syncthreads();
   }
+  __syncthreads();
   if (tid == 0 && gave_up) flag_error(p.status, OZK_ERR_TIMEOUT);
   if (singular && tid == 0 && rank == 0) flag_error(p.status, OZK_ERR_SINGULAR);
-  __syncthreads();
   for (int jl = cg; jl < ncol; jl += ng)
-    if (r < w) X[r + static_cast<long long>(dst[rank + C * jl]) * ldx] =
+    if (r < w) X[r + static_cast<long long>(dst[c0 + jl]) * ldx] =
         singular ? make_double2(0.0, 0.0) : A[static_cast<size_t>(jl) * max_w + r];
   // no CTA leaves while another may still send to it (every message is received before its step, but
   // a singular or abandoned block ends early)
@@ -829,24 +847,26 @@ void launch_tri_inv(const double2* T, long long ldt, int r, int upper, int unit,
 }
 
 void launch_gjinv(const GjParams& p, int max_w, int batch, cudaStream_t st) {
-  // A cluster per block while the launch leaves SMs idle: 8, 4 or 2 CTAs, as many as every block can
-  // have an SM for each.  64 x 64 blocks: 1 of them 135 us with 8 CTAs (350 in registers, 443 in
-  // shared memory by one CTA), 16 of them 190 us with 8 or 4, 38 of them 280 us with 2 or 4, 76 of
-  // them 280 us with 2; 152 of them 438 us with 2, so with more than an SM for every two blocks the
-  // one-CTA forms stay: the register form for blocks of order 56 < w <= 64 when every block of the
-  // launch has an SM to itself, the shared-memory kernel for the others.  Order 50: 106 us for one
-  // block with 8 CTAs against 275; order 112: 406 against 1831.  Which arithmetic inverts a block
-  // depends on its own order and on whether the launch has at most one block per SM only, so a block
-  // comes out the same alone and in a small batch.
+  // A cluster per block: 8 or 4 CTAs while every one can have an SM, 2 up to one block per SM (two CTAs
+  // an SM then, while their shared memory fits).  64 x 64 blocks: 1 of them 103 us with 8 CTAs (133 with
+  // 4, 221 with 2, 354 in registers by one CTA, 443 in shared memory), 16 of them 126 with 8, 133 with 4,
+  // 38 of them 195 with 4, 221 with 2, 76 of them 221 with 2 and 310 with 4, 152 of them 344 with 2 and
+  // 358 in registers, 256 of them 671 with 2 and 648 in shared memory: more than one block per SM take
+  // the one-CTA form.  Order 50: 83 us for one block with 8 CTAs against 262, 224 for 152 with 2 against
+  // 265; order 80: 170 for one against 739, 727 for 152 with 2 against 743; order 112: 348 against 1746.
+  // The register form is left for blocks of order 56 < w <= 64 beside wider ones.  Which arithmetic
+  // inverts a block depends on its own order and on whether the launch has at most one block per SM
+  // only, so a block comes out the same alone and in a batch of that size.
   const int sms = gpu_sm_count();
-  const int C = 8 * batch <= sms ? 8 : (4 * batch <= sms ? 4 : (2 * batch <= sms ? 2 : 1));
+  const bool two = 2 * batch <= sms || (batch <= sms && max_w <= 80);
+  const int C = 8 * batch <= sms ? 8 : (4 * batch <= sms ? 4 : (two ? 2 : 1));
   if (C > 1) {
     const size_t smem = sizeof(double2) * (static_cast<size_t>((max_w + C - 1) / C) * max_w +
                                            static_cast<size_t>(GJC_SLOTS) * (max_w + 2));
     cudaFuncSetAttribute(gjinv_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(static_cast<unsigned>(batch * C));
-    cfg.blockDim = dim3(GJINV_THREADS);
+    cfg.blockDim = dim3(GJC_THREADS);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];

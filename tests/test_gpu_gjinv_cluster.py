@@ -54,3 +54,19 @@ def test_singular_block_of_a_batch(ozk_mod, handle, batch):
     want = co.tau00_full(M, t0)
     for i in range(1, batch):
         assert kkr.rel_err(ozk_mod.to_numpy(taus[i]), want) < 1e-10, i
+
+
+@pytest.mark.parametrize("b,w", [(2, 2), (8, 64), (16, 80), (16, 96)])
+@pytest.mark.parametrize("batch", [100, 152])
+def test_two_clusters_an_sm(ozk_mod, handle, b, w, batch):
+    """More blocks than SM pairs: clusters of two CTAs share SMs up to order 80."""
+    Ms = [_matrix(b, w, 7 + i) for i in range(2)]
+    t0 = np.eye(b, dtype=np.complex128) * (0.3 + 0.1j)
+    dM = [ozk_mod.colmajor_cuda(Ms[i % 2]) for i in range(batch)]
+    dt = [ozk_mod.colmajor_cuda(t0) for _ in range(batch)]
+    taus = [ozk_mod.colmajor_cuda(np.zeros((b, b), dtype=np.complex128)) for _ in range(batch)]
+    ozk_mod.kkr_tau00_batched(handle, dM, dt, taus, S=8, nb=w)
+    assert handle.status() == 0
+    want = [co.tau00_full(M, t0) for M in Ms]
+    for i in range(batch):
+        assert kkr.rel_err(ozk_mod.to_numpy(taus[i]), want[i % 2]) < 1e-10, i
