@@ -317,7 +317,8 @@ ozk_status_t plan_gemm(const EmuGemm& g, GemmPlan* P) {
   P->offF = off; off = align_up(off + static_cast<size_t>(g.batch) * std::max(g.nmax, 1) * 4, 256);
   P->offT = off;                                                     // tile prefix sums
   off = align_up(off + (static_cast<size_t>(std::max(g.batch, g.gbatch)) + 1) * 4, 256);
-  // row maxima of the K-parallel split (left, right operand)
+  // 8 bytes per row of either operand, unused since a split's row maxima stay in the CTAs' shared
+  // memory: kept, so that a call needs the scratch that it always did
   P->offGA = off; off = align_up(off + static_cast<size_t>(g.batch) * P->rowsA * 8, 256);
   P->offGB = off; off = align_up(off + static_cast<size_t>(g.batch) * std::max(g.nmax, 1) * 8, 256);
   // split K: a single problem whose tiles fill less than half of the SMs and whose K spans

@@ -4,7 +4,8 @@
 //                        batch of small blocks (D up to 64 x 64): R = I gives D^-1 (the
 //                        pivot-block inverse of the block LU), R = t_0 gives S_00^-1 t_0.
 //   * gjinv_kernel     : in-place Gauss-Jordan inversion with partial pivoting of pivot blocks
-//                        up to 112 x 112 (the panel's D^-1 of the block LU).
+//                        up to 112 x 112 (the panel's D^-1 of the block LU); gjinv_cluster_kernel
+//                        spreads each block over 8, 4 or 2 CTAs, gjinv_reg_kernel holds it in registers.
 //   * build_m_kernel   : M = I - blockdiag(t) G.
 //   * scale_kernel     : C = beta C (the k == 0 / alpha == 0 case of the GEMM API).
 // These are the only places with O(n b^2) / O(n^2 b) binary64 arithmetic of the solve.
@@ -334,8 +335,8 @@ gjinv_kernel(const GjParams p, int skip_lo, int skip_hi) {
 // w^3 complex multiply-adds per block, as in gjinv_kernel; 350 against 423 us per 64 x 64
 // block on one SM.  Its 128 registers a thread fill half of an SM's register file, so two
 // such CTAs on one SM leave no room for the side stream's split CTAs that run beside the
-// shared-memory kernel: it serves launches of at most one block per SM that are too many for clusters.  Rows at or beyond w
-// are skipped, but a warp spans 32 columns whatever w is, so narrower blocks (w = 48: 3/4 of
+// shared-memory kernel: it serves launches of at most one block per SM, where clusters of two do
+// not fit (blocks of order above 80 in the launch).  Rows at or beyond w are skipped, but a warp spans 32 columns whatever w is, so narrower blocks (w = 48: 3/4 of
 // the lanes busy) stay with the shared-memory kernel.
 constexpr int GJR_THREADS = 256;
 constexpr int GJR_W = 64;
@@ -479,7 +480,8 @@ gjinv_reg_kernel(const GjParams p) {
 // takes, column k + 1, |.|^2 and the division one after the other), and one block of a launch has the whole GPU: the one-CTA forms (block in shared
 // memory: 423 us; in registers: 350 us) left 7/8 or more of it idle in single solves and small
 // batches.  With the columns dealt round robin, so that every step's message crossed between CTAs on
-// the chain, and sent as 16-byte stores (st.async: about 8 clocks each, 528 a step), 8 CTAs took 135 us.  C and the figures of each: launch_gjinv.
+// the chain, and sent as 528 16-byte stores, 8 CTAs took 135 us (103 now).  C and the figures of each:
+// launch_gjinv.
 // Same operations on every element as the one-CTA form of the block's order, so a block comes out the
 // same in a launch of any size up to one block per SM; `from_zero`: column k of the inverse by the
 // multiply-adds of the elimination applied to zero (gjinv_reg_kernel) instead of the negated product.

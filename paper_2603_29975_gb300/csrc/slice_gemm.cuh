@@ -8,11 +8,14 @@
 //   * warp 0 (one lane) streams K-blocks of 16 with TMA: one box of two halves of S slices of A
 //     (128 rows) and one of B (BN rows) per pipeline stage, in runs of 2 KB and BN x 16 bytes, which
 //     land as the unswizzled core-matrix layout of the MMA descriptors;
-//   * warp 1 (one lane) issues tcgen05.mma kind::f16 for every pair (s, t) of the pair set,
+//   * warp 1 (one elected lane) issues tcgen05.mma kind::f16 for every pair (s, t) of the pair set,
 //     accumulating pair products of the same weight class g = s + t into one FP32 TMEM
-//     accumulator per group (G groups x BN columns of the 512); after a chunk's first K-block
-//     the partners of each A slice share one MMA over the stacked B slices;
-//   * warps 2..17 drain the accumulators.  Every product of two digits is an integer of
+//     accumulator per group (G groups x BN columns of the 512); where the groups are accumulated
+//     already, the partners of each A slice share one MMA over the stacked B slices, and around a
+//     chunk's boundary the groups go in two parts, so that one part is drained while the tensor
+//     cores work on the other;
+//   * warp 2 finds the CTA's tiles ahead of the others and leaves them in a ring;
+//   * warps 4..19 drain the accumulators.  Every product of two digits is an integer of
 //     magnitude <= 2^14 and each accumulator receives at most 1024 of them per "exactness
 //     chunk" of K, so every FP32 value is an exact integer <= 2^24.  The epilogue converts
 //     it to int32 and adds it, shifted by its group weight 8 (g_max - g) bits, into a 64-bit
@@ -32,7 +35,7 @@ namespace ozk {
 
 constexpr int GEMM_BM = 128;
 constexpr int GEMM_EPI_WARPS = 16;
-// warpgroup 0 (warps 0..3): TMA producer (warp 0), MMA issuer (warp 1), two idle warps; it
+// warpgroup 0 (warps 0..3): TMA producer (warp 0), MMA issuer (warp 1), tiles (warp 2), an idle warp; it
 // hands registers to the four epilogue warpgroups (setmaxnreg), whose exact sums of 16 outputs
 // need more than the 96 registers a thread of a 20-warp CTA starts with
 constexpr int GEMM_CTRL_WARPS = 4;
