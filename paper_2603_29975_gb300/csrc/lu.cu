@@ -515,6 +515,7 @@ gjinv_cluster_kernel(const GjParams p, int C, int max_w) {
   __shared__ int wrow[4];
   __shared__ int dst[GJINV_MAX];            // column j of the block is column dst[j] of X
   __shared__ int gave_up;                   // 1 + the first step whose message did not come
+  grid_dependency_wait();                   // the kernels that wrote the block and the tables
   const int z = blockIdx.x / C, rank = blockIdx.x % C;
   const bool single = p.D == nullptr;
   const int w = single ? p.nb1 : p.nb[z];
@@ -871,13 +872,14 @@ void launch_gjinv(const GjParams& p, int max_w, int batch, cudaStream_t st) {
     cfg.blockDim = dim3(GJC_THREADS);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = static_cast<unsigned>(C);
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1] = pdl_attribute();
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     cudaLaunchKernelEx(&cfg, gjinv_cluster_kernel, p, C, max_w);
     record_launch();
     return;

@@ -122,6 +122,14 @@ __device__ __forceinline__ void mbar_fence_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
+// Programmatic dependent launch: a kernel launched with pdl_attribute() may start while the kernel before
+// it in the stream ends (its launch and prologue overlap that kernel's last CTAs); every CTA calls
+// grid_dependency_wait() before it touches memory that another kernel writes or reads, which returns
+// when that kernel is complete and its writes are visible.  launch_dependents() lets the next kernel's
+// CTAs come as soon as every CTA of this one has called it, instead of at their ends.
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_u32(bar)) : "memory");
 }

@@ -134,6 +134,12 @@ void launch_tile_prefix(const GemmParams& p, int BN, int batch, int* out, cudaSt
 // (the modes of the slice GEMM's epilogue: store, LU, general)
 void launch_finish_split(const GemmParams& p, cudaStream_t st);
 int gpu_sm_count();
+inline cudaLaunchAttribute pdl_attribute() {
+  cudaLaunchAttribute a{};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  return a;
+}
 // operand stages (K-blocks of 16 in flight) of a CTA, 0: none fits
 int gemm_stages(int S, int BN);
 

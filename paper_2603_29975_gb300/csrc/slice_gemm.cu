@@ -73,6 +73,7 @@ __global__ void __launch_bounds__(256) finish_split_kernel(const __grid_constant
   constexpr int NH = G < 4 ? G : 4;
   constexpr int NL = G - NH;
   constexpr int S8 = 8 * NL;
+  grid_dependency_wait();
   const int m = p.m1, n = p.n1, n2 = 2 * n;
   const long long total = static_cast<long long>(m) * n;
   for (long long idx = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; idx < total;
@@ -113,15 +114,22 @@ __global__ void __launch_bounds__(256) finish_split_kernel(const __grid_constant
 void launch_finish_split(const GemmParams& p, cudaStream_t st) {
   const long long total = static_cast<long long>(p.m1) * p.n1;
   const unsigned blocks = static_cast<unsigned>(std::min<long long>((total + 255) / 256, 8L * num_sms()));
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1] = {pdl_attribute()};
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
   switch (p.ngroups) {
-    case 1: finish_split_kernel<1><<<blocks, 256, 0, st>>>(p); break;
-    case 2: finish_split_kernel<2><<<blocks, 256, 0, st>>>(p); break;
-    case 3: finish_split_kernel<3><<<blocks, 256, 0, st>>>(p); break;
-    case 4: finish_split_kernel<4><<<blocks, 256, 0, st>>>(p); break;
-    case 5: finish_split_kernel<5><<<blocks, 256, 0, st>>>(p); break;
-    case 6: finish_split_kernel<6><<<blocks, 256, 0, st>>>(p); break;
-    case 7: finish_split_kernel<7><<<blocks, 256, 0, st>>>(p); break;
-    default: finish_split_kernel<8><<<blocks, 256, 0, st>>>(p); break;
+    case 1: cudaLaunchKernelEx(&cfg, finish_split_kernel<1>, p); break;
+    case 2: cudaLaunchKernelEx(&cfg, finish_split_kernel<2>, p); break;
+    case 3: cudaLaunchKernelEx(&cfg, finish_split_kernel<3>, p); break;
+    case 4: cudaLaunchKernelEx(&cfg, finish_split_kernel<4>, p); break;
+    case 5: cudaLaunchKernelEx(&cfg, finish_split_kernel<5>, p); break;
+    case 6: cudaLaunchKernelEx(&cfg, finish_split_kernel<6>, p); break;
+    case 7: cudaLaunchKernelEx(&cfg, finish_split_kernel<7>, p); break;
+    default: cudaLaunchKernelEx(&cfg, finish_split_kernel<8>, p); break;
   }
   record_launch();
 }

@@ -769,6 +769,7 @@ slice_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_holder;
+  grid_dependency_wait();                      // the operands' split; C, exponents and tables of kernels before it
   if (p.stall_cycles > 0) {
     // failure-path test: one thread's bounded wait runs out (OZK_ERR_TIMEOUT, abort flag set)
     // before any TMA copy or MMA has been issued; every role then skips its loop
@@ -1178,7 +1179,15 @@ inline void launch_instance(const CUtensorMap& ta, const CUtensorMap& tb, const 
                             cudaStream_t st) {
   cudaFuncSetAttribute(slice_gemm_kernel<BN, SF, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        static_cast<int>(smem));
-  slice_gemm_kernel<BN, SF, KS><<<grid, GEMM_THREADS, smem, st>>>(ta, tb, p);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(grid));
+  cfg.blockDim = dim3(GEMM_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1] = {pdl_attribute()};
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, slice_gemm_kernel<BN, SF, KS>, ta, tb, p);
 }
 // the instances of S = 3..5, of S = 6..8 (split K: S = 7) and of S = 9, 10, each in its own
 // translation unit

@@ -388,6 +388,8 @@ template <int SF, bool W64>
 __global__ void __launch_bounds__(SPLIT_MAX_WARPS * 32, 2) split_kernel(const __grid_constant__ SplitPair pp) {
   __shared__ unsigned long long wmax[SPLIT_MAX_WARPS][SPLIT_ROWS];     // row maxima of the warps
   __shared__ unsigned long long cmax[SPLIT_MAX_KG][SPLIT_ROWS];        // and of the cluster's CTAs
+  grid_dependency_wait();
+  launch_dependents();
   if (pp.s[blockIdx.z].side == 0) split_rows<SF, W64, 0>(pp.s[blockIdx.z], wmax, cmax);
   else split_rows<SF, W64, 1>(pp.s[blockIdx.z], wmax, cmax);
 }
@@ -415,13 +417,14 @@ void launch_split(const SplitParams& a, int rows_a, const SplitParams* b, int ro
   cfg.gridDim = dim3(static_cast<unsigned>(rblocks * kg), static_cast<unsigned>(batch), static_cast<unsigned>(pp.nsides));
   cfg.blockDim = dim3(32u * static_cast<unsigned>(std::max(std::min(share, SPLIT_MAX_WARPS), kg)));
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = static_cast<unsigned>(kg);
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = kg > 1 ? 1 : 0;
+  at[1] = pdl_attribute();
+  cfg.attrs = kg > 1 ? at : at + 1;
+  cfg.numAttrs = kg > 1 ? 2 : 1;
   // compile-time slice counts 3..10 (nbits = 8 S - 1 on every side); the test hook's digit copy and
   // other slice counts take the run-time form
   int sf = pp.s[0].S;
