@@ -1091,8 +1091,9 @@ namespace ozk {
 // D^-1 into the solve's nb x nb slot of dinv), GEMM 1 (L = M[0:p, p:q] D^-1, in place) and GEMM 2
 // (M[0:p, 0:p] -= L M[p:q, 0:p]); step < 0 the final S_00 solve.  Finished solves get zero
 // sizes.
-__global__ void kkr_step_kernel(int panel, int leaf, int nleaves, int nsolves, const int* __restrict__ n,
-                                double2* const* M, int b, int W, int w, double2* dinv, KkrStep t) {
+__global__ void kkr_step_kernel(int panel, int leaf, int nleaves, int nsolves, const int* n, double2* const* M, int b,
+                                int W, int w, double2* dinv, KkrStep t) {
+  grid_dependency_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nsolves) return;
   const int ni = n[i];
@@ -1129,7 +1130,7 @@ __global__ void kkr_step_kernel(int panel, int leaf, int nleaves, int nsolves, c
 
 void launch_kkr_step(int panel, int leaf, int nleaves, int nsolves, const int* n, double2* const* M, int b, int W,
                      int w, double2* dinv, const KkrStep& t, cudaStream_t st) {
-  kkr_step_kernel<<<(nsolves + 127) / 128, 128, 0, st>>>(panel, leaf, nleaves, nsolves, n, M, b, W, w, dinv, t);
+  launch_pdl(kkr_step_kernel, (nsolves + 127) / 128, 128, st, panel, leaf, nleaves, nsolves, n, M, b, W, w, dinv, t);
   record_launch();
 }
 

@@ -140,6 +140,18 @@ inline cudaLaunchAttribute pdl_attribute() {
   a.val.programmaticStreamSerializationAllowed = 1;
   return a;
 }
+// k<<<g, b, 0, st>>>(args...) with that attribute; k starts with grid_dependency_wait()
+template <typename... P, typename... A>
+void launch_pdl(void (*k)(P...), dim3 g, dim3 b, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = g;
+  cfg.blockDim = b;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1] = {pdl_attribute()};
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
 // operand stages (K-blocks of 16 in flight) of a CTA, 0: none fits
 int gemm_stages(int S, int BN);
 

@@ -51,6 +51,7 @@ __device__ __forceinline__ double sm_uniform(uint64_t base, uint64_t idx) {
 // X (n x SEL_PROBES, column major): Re of column p from stream 2p, Im from stream 2p + 1,
 // (U - 1/2) * sqrt(6), so that every entry has E|x|^2 = 1.
 __global__ void probe_kernel(double2* X, int n, SelBases bases) {
+  grid_dependency_wait();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   const double c = 2.449489742783178;   // sqrt(6) rounded to binary64
@@ -108,6 +109,7 @@ __device__ __forceinline__ double crest_of(double r, int e, double sh, int len) 
 constexpr int VS_ROWS = 16, VS_LANES = 32;
 __global__ void __launch_bounds__(VS_ROWS * VS_LANES)
 vec_stats_rows_kernel(const double2* M, long long ld, int count, int len, SelVecStats out) {
+  grid_dependency_wait();
   __shared__ unsigned long long smax[VS_LANES][VS_ROWS];
   __shared__ double ssum[VS_LANES][VS_ROWS];
   __shared__ int sz[VS_LANES][VS_ROWS];
@@ -159,6 +161,7 @@ vec_stats_rows_kernel(const double2* M, long long ld, int count, int len, SelVec
 // of the kernel's 33 us at 1536 vectors of 192)
 __global__ void __launch_bounds__(256)
 vec_stats_cols_kernel(const double2* M, long long ld, int count, int len, SelVecStats out) {
+  grid_dependency_wait();
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   __shared__ double fr[8], fsh[8];
@@ -201,6 +204,7 @@ vec_stats_cols_kernel(const double2* M, long long ld, int count, int len, SelVec
 
 // EA = max e over the nonzero rows of op(A), EB likewise over op(B)'s columns (0 if none).
 __global__ void __launch_bounds__(1024) max_exp_kernel(SelVecStats a, int ma, SelVecStats b, int nb, int* ex) {
+  grid_dependency_wait();
   __shared__ int sa[32], sb[32];
   int xa = INT_MIN, xb = INT_MIN;
   // r is non-negative: r > 0 by its bits
@@ -292,6 +296,7 @@ constexpr int GEMV_CHUNK = 16;
 template <bool PLAIN, int NP>
 __global__ void gemv_rows_kernel(const double2* M, long long ld, int rows, int len, const double2* Xh,
                                  const double2* Xl, int ldx, double2* part, const int* ex, int eidx) {
+  grid_dependency_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= rows) return;
   const Pow2 s = ex ? pow2_neg(ex[eidx]) : Pow2{1.0, 1.0};
@@ -329,6 +334,7 @@ __global__ void gemv_rows_kernel(const double2* M, long long ld, int rows, int l
 // its 8 additions in the shuffles' tree, every one of 32 lanes wide on the FP64 pipe: 44 us for 6144
 // outputs of 96 chunks); CTAs of two warps, so that the few outputs of a short operand use more SMs
 __global__ void gemv_reduce_kernel(const double2* part, int rows, int nchunks, double2* Yh, double2* Yl) {
+  grid_dependency_wait();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31, sub = lane >> 3;
   const int idx = (t >> 5) * 8 + (lane & 7);
@@ -355,6 +361,7 @@ __global__ void gemv_reduce_kernel(const double2* part, int rows, int nchunks, d
 __global__ void gemv_cols_kernel(const double2* M, long long ld, int rows, int len, int conj, const double2* Xh,
                                  const double2* Xl, int ldx, double2* Yh, double2* Yl, int ldy, const int* ex,
                                  int eidx) {
+  grid_dependency_wait();
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (w >= rows) return;
@@ -508,6 +515,7 @@ __device__ CrestPart crest_merge(const CrestPart* parts, int lane) {
 __global__ void __cluster_dims__(FEAT_C, 1, 1) __launch_bounds__(FEAT_T)
 selector_features_kernel(SelVecStats a, int m, SelVecStats b, int n, int k, const double2* X, const double2* zs,
                          const int* ex, float* f, SelAux* aux) {
+  grid_dependency_wait();
   // zs: the leading parts of the double-double probe product
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
@@ -628,6 +636,7 @@ selector_features_kernel(SelVecStats a, int m, SelVecStats b, int n, int k, cons
 // (block partials of num and den into rpart, then residual_final_kernel sums them in order)
 __global__ void __launch_bounds__(RED_T) residual_kernel(const double2* Wh, const double2* Wl, const double2* zh,
                                                          const double2* zl, int m, SelAux* aux, double* rpart) {
+  grid_dependency_wait();
   __shared__ double sh[RED_T];
   const int E = aux->E;
   double num = 0, den = 0;
@@ -649,6 +658,7 @@ __global__ void __launch_bounds__(RED_T) residual_kernel(const double2* Wh, cons
 }
 
 __global__ void __launch_bounds__(RED_T) residual_final_kernel(const double* rpart, int nblocks, SelAux* aux) {
+  grid_dependency_wait();
   __shared__ double sh[RED_T];
   double num = 0, den = 0;
   for (int b = threadIdx.x; b < nblocks; b += RED_T) {
@@ -722,6 +732,7 @@ __device__ __forceinline__ void load_params(const float* P, float* w) {
 // same bits): one thread through all three layers took 21 us for the one sample of a prediction.
 __global__ void __launch_bounds__(SEL_NH) mlp_forward_few_kernel(const float* P, const float* X, float* Z1, float* Z2,
                                                                  float* Y) {
+  grid_dependency_wait();
   __shared__ float h1[SEL_NH], h2[SEL_NH];
   const int s = blockIdx.x, j = threadIdx.x;
   float z = P[OFF_B1 + j];
@@ -862,6 +873,7 @@ __global__ void __launch_bounds__(RED_T) mse_kernel(const float* Y, const float*
 
 // smallest S in 3..10 with prediction <= lim, else 10; aux->S and the predictions
 __global__ void choose_kernel(const float* Y, float lim, SelAux* aux) {
+  grid_dependency_wait();
   if (threadIdx.x) return;
   int S = SEL_SMAX;
   for (int o = 0; o < SEL_NO; ++o) {
@@ -886,7 +898,7 @@ __global__ void defer_check_kernel(const SelAux* aux, int S, int with_pred, doub
 static unsigned blocks(long long n, int t) { return static_cast<unsigned>((n + t - 1) / t); }
 
 void launch_probe(double2* X, int n, const SelBases& b, cudaStream_t st) {
-  probe_kernel<<<blocks(n, 256), 256, 0, st>>>(X, n, b);
+  launch_pdl(probe_kernel, blocks(n, 256), 256, st, X, n, b);
   record_launch();
 }
 
@@ -894,14 +906,14 @@ void launch_vec_stats(const double2* M, long long ld, int count, int len, bool c
                       cudaStream_t st) {
   if (count <= 0) return;
   if (contiguous)
-    vec_stats_cols_kernel<<<blocks(static_cast<long long>(count) * 32, 256), 256, 0, st>>>(M, ld, count, len, out);
+    launch_pdl(vec_stats_cols_kernel, blocks(static_cast<long long>(count) * 32, 256), 256, st, M, ld, count, len, out);
   else
-    vec_stats_rows_kernel<<<blocks(count, VS_ROWS), VS_ROWS * VS_LANES, 0, st>>>(M, ld, count, len, out);
+    launch_pdl(vec_stats_rows_kernel, blocks(count, VS_ROWS), VS_ROWS * VS_LANES, st, M, ld, count, len, out);
   record_launch();
 }
 
 void launch_max_exp(const SelVecStats& a, int ma, const SelVecStats& b, int nb, int* ex, cudaStream_t st) {
-  max_exp_kernel<<<1, 1024, 0, st>>>(a, ma, b, nb, ex);
+  launch_pdl(max_exp_kernel, 1, 1024, st, a, ma, b, nb, ex);
   record_launch();
 }
 
@@ -914,33 +926,33 @@ void launch_gemv(const double2* M, long long ld, int rows, int len, int op, cons
   if (op == 0) {
     const int nch = std::max(1, gemv_chunks(len));
     if (plain)
-      gemv_rows_kernel<true, SEL_PROBES><<<dim3(blocks(rows, 64), nch, 1), 64, 0, st>>>(M, ld, rows, len, Xh, Xl, ldx,
-                                                                                        part, ex, eidx);
+      launch_pdl(gemv_rows_kernel<true, SEL_PROBES>, dim3(blocks(rows, 64), nch, 1), 64, st, M, ld, rows, len, Xh, Xl,
+                 ldx, part, ex, eidx);
     else
-      gemv_rows_kernel<false, 1><<<dim3(blocks(rows, 64), nch, SEL_PROBES), 64, 0, st>>>(M, ld, rows, len, Xh, Xl, ldx,
-                                                                                         part, ex, eidx);
+      launch_pdl(gemv_rows_kernel<false, 1>, dim3(blocks(rows, 64), nch, SEL_PROBES), 64, st, M, ld, rows, len, Xh, Xl,
+                 ldx, part, ex, eidx);
     record_launch();
-    gemv_reduce_kernel<<<blocks((static_cast<long long>(rows) * SEL_PROBES + 7) / 8 * 32, 64), 64, 0, st>>>(
-        part, rows, nch, Yh, Yl);
+    launch_pdl(gemv_reduce_kernel, blocks((static_cast<long long>(rows) * SEL_PROBES + 7) / 8 * 32, 64), 64, st, part,
+               rows, nch, Yh, Yl);
   } else {
-    gemv_cols_kernel<<<blocks(static_cast<long long>(rows) * 32, 256), 256, 0, st>>>(M, ld, rows, len, op == 2, Xh,
-                                                                                     Xl, ldx, Yh, Yl, rows, ex, eidx);
+    launch_pdl(gemv_cols_kernel, blocks(static_cast<long long>(rows) * 32, 256), 256, st, M, ld, rows, len, op == 2, Xh,
+               Xl, ldx, Yh, Yl, rows, ex, eidx);
   }
   record_launch();
 }
 
 void launch_selector_features(const SelVecStats& a, int m, const SelVecStats& b, int n, int k, const double2* X,
                               const double2* zs, const int* ex, float* f, SelAux* aux, cudaStream_t st) {
-  selector_features_kernel<<<FEAT_C, FEAT_T, 0, st>>>(a, m, b, n, k, X, zs, ex, f, aux);
+  launch_pdl(selector_features_kernel, FEAT_C, FEAT_T, st, a, m, b, n, k, X, zs, ex, f, aux);
   record_launch();
 }
 
 void launch_residual(const double2* Wh, const double2* Wl, const double2* zh, const double2* zl, int m, SelAux* aux,
                      double* rpart, cudaStream_t st) {
   const int nb = static_cast<int>(std::min<long long>(256, blocks(static_cast<long long>(m) * SEL_PROBES, RED_T)));
-  residual_kernel<<<nb, RED_T, 0, st>>>(Wh, Wl, zh, zl, m, aux, rpart);
+  launch_pdl(residual_kernel, nb, RED_T, st, Wh, Wl, zh, zl, m, aux, rpart);
   record_launch();
-  residual_final_kernel<<<1, RED_T, 0, st>>>(rpart, nb, aux);
+  launch_pdl(residual_final_kernel, 1, RED_T, st, rpart, nb, aux);
   record_launch();
 }
 
@@ -963,7 +975,7 @@ void launch_axpby(int m, int n, const double2* D, long long ldd, double2* C, lon
 void launch_mlp_forward(const float* P, const float* X, int N, float* Z1, float* Z2, float* Y, cudaStream_t st) {
   if (N <= 0) return;
   // a CTA a sample while the samples fit the SMs
-  if (N <= gpu_sm_count()) mlp_forward_few_kernel<<<N, SEL_NH, 0, st>>>(P, X, Z1, Z2, Y);
+  if (N <= gpu_sm_count()) launch_pdl(mlp_forward_few_kernel, N, SEL_NH, st, P, X, Z1, Z2, Y);
   else mlp_forward_kernel<<<blocks(N, 128), 128, 0, st>>>(P, X, N, Z1, Z2, Y);
   record_launch();
 }
@@ -1005,7 +1017,7 @@ void launch_log_err(const double* rel, float* dst, cudaStream_t st) {
 }
 
 void launch_choose(const float* Y, float lim, SelAux* aux, cudaStream_t st) {
-  choose_kernel<<<1, 32, 0, st>>>(Y, lim, aux);
+  launch_pdl(choose_kernel, 1, 32, st, Y, lim, aux);
   record_launch();
 }
 

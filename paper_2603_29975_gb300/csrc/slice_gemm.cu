@@ -136,9 +136,9 @@ void launch_finish_split(const GemmParams& p, cudaStream_t st) {
 
 // Tile counts of the problems of a batched GEMM (each over its own grid, tiles wholly inside
 // its skip box left out) and their exclusive prefix sums: one CTA, chunks of 1024 problems.
-__global__ void __launch_bounds__(1024) tile_prefix_kernel(const int* __restrict__ m, const int* __restrict__ n,
-                                                           const int* __restrict__ skm, const int* __restrict__ skn,
-                                                           int batch, int BN, int* __restrict__ out) {
+__global__ void __launch_bounds__(1024) tile_prefix_kernel(const int* m, const int* n, const int* skm, const int* skn,
+                                                           int batch, int BN, int* out) {
+  grid_dependency_wait();
   __shared__ int part[1024];
   __shared__ int carry;
   if (threadIdx.x == 0) carry = 0;
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(1024) tile_prefix_kernel(const int* __restrict
 }
 
 void launch_tile_prefix(const GemmParams& p, int BN, int batch, int* out, cudaStream_t st) {
-  tile_prefix_kernel<<<1, 1024, 0, st>>>(p.m, p.n, p.skm, p.skn, batch, BN, out);
+  launch_pdl(tile_prefix_kernel, 1, 1024, st, p.m, p.n, p.skm, p.skn, batch, BN, out);
   record_launch();
 }
 
