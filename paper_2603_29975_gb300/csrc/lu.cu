@@ -877,7 +877,7 @@ void launch_gjinv(const GjParams& p, int max_w, int batch, cudaStream_t st) {
     at[0].val.clusterDim.x = static_cast<unsigned>(C);
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
-    at[1] = pdl_attribute();
+    at[1] = pdl_attribute(st);
     cfg.attrs = at;
     cfg.numAttrs = 2;
     cudaLaunchKernelEx(&cfg, gjinv_cluster_kernel, p, C, max_w);

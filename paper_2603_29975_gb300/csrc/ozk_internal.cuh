@@ -122,7 +122,7 @@ __device__ __forceinline__ void mbar_fence_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
-// Programmatic dependent launch: a kernel launched with pdl_attribute() may start while the kernel before
+// Programmatic dependent launch: a kernel launched with pdl_attribute may start while the kernel before
 // it in the stream ends (its launch and prologue overlap that kernel's last CTAs); every CTA calls
 // grid_dependency_wait() before it touches memory that another kernel writes or reads, which returns
 // when that kernel is complete and its writes are visible.  launch_dependents() lets the next kernel's

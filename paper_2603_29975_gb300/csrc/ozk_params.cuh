@@ -134,10 +134,14 @@ void launch_tile_prefix(const GemmParams& p, int BN, int batch, int* out, cudaSt
 // (the modes of the slice GEMM's epilogue: store, LU, general)
 void launch_finish_split(const GemmParams& p, cudaStream_t st);
 int gpu_sm_count();
-inline cudaLaunchAttribute pdl_attribute() {
+// not in a captured launch: replayed from a graph, the 256-solve step took 149.8 ms with such edges and
+// 143.6 without (its branches: pivot inverses beside the side stream's splits)
+inline cudaLaunchAttribute pdl_attribute(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool known = cudaStreamIsCapturing(st, &cap) == cudaSuccess;
   cudaLaunchAttribute a{};
   a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  a.val.programmaticStreamSerializationAllowed = 1;
+  a.val.programmaticStreamSerializationAllowed = known && cap == cudaStreamCaptureStatusNone ? 1 : 0;
   return a;
 }
 // k<<<g, b, 0, st>>>(args...) with that attribute; k starts with grid_dependency_wait()
@@ -147,7 +151,7 @@ void launch_pdl(void (*k)(P...), dim3 g, dim3 b, cudaStream_t st, A... args) {
   cfg.gridDim = g;
   cfg.blockDim = b;
   cfg.stream = st;
-  cudaLaunchAttribute at[1] = {pdl_attribute()};
+  cudaLaunchAttribute at[1] = {pdl_attribute(st)};
   cfg.attrs = at;
   cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);

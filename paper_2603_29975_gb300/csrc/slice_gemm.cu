@@ -118,7 +118,7 @@ void launch_finish_split(const GemmParams& p, cudaStream_t st) {
   cfg.gridDim = dim3(blocks);
   cfg.blockDim = dim3(256);
   cfg.stream = st;
-  cudaLaunchAttribute at[1] = {pdl_attribute()};
+  cudaLaunchAttribute at[1] = {pdl_attribute(st)};
   cfg.attrs = at;
   cfg.numAttrs = 1;
   switch (p.ngroups) {

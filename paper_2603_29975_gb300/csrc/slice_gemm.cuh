@@ -1184,7 +1184,7 @@ inline void launch_instance(const CUtensorMap& ta, const CUtensorMap& tb, const 
   cfg.blockDim = dim3(GEMM_THREADS);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1] = {pdl_attribute()};
+  cudaLaunchAttribute at[1] = {pdl_attribute(st)};
   cfg.attrs = at;
   cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, slice_gemm_kernel<BN, SF, KS>, ta, tb, p);

@@ -422,7 +422,7 @@ void launch_split(const SplitParams& a, int rows_a, const SplitParams* b, int ro
   at[0].val.clusterDim.x = static_cast<unsigned>(kg);
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
-  at[1] = pdl_attribute();
+  at[1] = pdl_attribute(st);
   cfg.attrs = kg > 1 ? at : at + 1;
   cfg.numAttrs = kg > 1 ? 2 : 1;
   // compile-time slice counts 3..10 (nbits = 8 S - 1 on every side); the test hook's digit copy and
