@@ -397,7 +397,6 @@ __device__ __forceinline__ bool release_unread(uint64_t* acc_empty, ChunkWait& c
       __syncwarp();
       if (lane == 0) mbar_arrive(&acc_empty[gi]);
     }
-    if (G <= split_group(G) && !cw.part(1)) return false;
   }
   return true;
 }
@@ -470,12 +469,14 @@ __device__ __forceinline__ void fold_steps(const EpiCtx& x, uint64_t* acc_empty,
     fold_steps<G, NH, I + 1, GE, REDO>(x, acc_empty, lane, early, big, H, L);
   }
 }
-// Groups [G0, GE) of one chunk (a part of the accumulators).
+// Groups [G0, GE) of one chunk (a part of the accumulators).  A part without groups (the second one
+// of G = 1) is not waited for: nothing it releases would hold the issuer back, which could complete
+// that barrier's phase of the next chunk too before a slow warp had seen this one's.
 template <int G, int NH, int G0, int GE>
 __device__ __forceinline__ bool fold_part(const EpiCtx& x, uint64_t* acc_empty, int lane, uint32_t magic_mask,
                                           ChunkWait& cw, unsigned long long (&H)[16], unsigned long long (&L)[16]) {
-  if (!cw.part(G0 == 0 ? 0 : 1)) return false;
   if constexpr (G0 < GE) {
+    if (!cw.part(G0 == 0 ? 0 : 1)) return false;
     constexpr int I0 = FoldPlan<G, NH>::first_step(G0);
     constexpr uint32_t need = ((1u << (GE - G0)) - 1u) << G0;
     const bool known = (magic_mask & need) == need;
