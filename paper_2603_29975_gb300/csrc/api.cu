@@ -317,8 +317,7 @@ ozk_status_t plan_gemm(const EmuGemm& g, GemmPlan* P) {
   P->offF = off; off = align_up(off + static_cast<size_t>(g.batch) * std::max(g.nmax, 1) * 4, 256);
   P->offT = off;                                                     // tile prefix sums
   off = align_up(off + (static_cast<size_t>(std::max(g.batch, g.gbatch)) + 1) * 4, 256);
-  // 8 bytes per row of either operand, unused since a split's row maxima stay in the CTAs' shared
-  // memory: kept, so that a call needs the scratch that it always did
+  // row maxima of either operand (splits of few row blocks with a long K)
   P->offGA = off; off = align_up(off + static_cast<size_t>(g.batch) * P->rowsA * 8, 256);
   P->offGB = off; off = align_up(off + static_cast<size_t>(g.batch) * std::max(g.nmax, 1) * 8, 256);
   // split K: a single problem whose tiles fill less than half of the SMs and whose K spans
@@ -369,6 +368,7 @@ ozk_status_t run_emulated(ozk_context* h, const EmuGemm& g, size_t ws_offset = 0
   sp.trans = g.oa.trans; sp.conj = g.oa.conj; sp.side = 0;
   sp.out_rows = P.rowsA; sp.out = As; sp.exps = e; sp.exp_stride = P.rowsA;
   sp.dbg_digits = g.dbg_digits_a;
+  sp.gmax = reinterpret_cast<unsigned long long*>(ws + P.offGA);
   if (single) { sp.X = nullptr; sp.X1 = g.A; sp.ld1 = g.lda; sp.rows1 = g.m; sp.k1 = g.k; sp.zstride1 = g.zsA; }
   else { sp.X = g.tA; sp.ld = g.tlda; sp.rows = g.tm; sp.kdim = g.tk; }
   const double smnk = g.sum_mnk >= 0 ? g.sum_mnk : static_cast<double>(g.m) * g.n * g.k;
@@ -379,6 +379,7 @@ ozk_status_t run_emulated(ozk_context* h, const EmuGemm& g, size_t ws_offset = 0
   sq.trans = g.ob.trans ? 0 : 1; sq.conj = g.ob.conj; sq.side = 1;
   sq.out_rows = P.rowsB; sq.out = Bs; sq.exps = f; sq.exp_stride = std::max(g.nmax, 1);
   sq.dbg_digits = nullptr;
+  sq.gmax = reinterpret_cast<unsigned long long*>(ws + P.offGB);
   if (single) { sq.X = nullptr; sq.X1 = g.B; sq.ld1 = g.ldb; sq.rows1 = g.n; sq.k1 = g.k; sq.zstride1 = g.zsB; }
   else { sq.X = g.tB; sq.ld = g.tldb; sq.rows = g.tn; sq.kdim = g.tk; }
   const bool split_a = (g.split_sides & 1) != 0, split_b = (g.split_sides & 2) != 0;

@@ -27,7 +27,10 @@ struct SplitParams {
   // uniform batch starts at X1 + z * zstride1
   const double2* X1; int ld1, rows1, k1;
   long long zstride1;
-  int kgroups;              // CTAs (a cluster) that share a row block's K-blocks (set by the launcher)
+  int kgroups;              // CTAs that share a row block's K-blocks (set by the launcher)
+  // [batch][exp_stride] scratch for the rows' largest |Re|, |Im| bit patterns (few row blocks, long K);
+  // the launcher clears it, or passes null where the splitting CTAs find the maxima themselves
+  unsigned long long* gmax;
 };
 struct SplitPair { SplitParams s[2]; int nsides; };
 

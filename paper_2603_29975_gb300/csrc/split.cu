@@ -25,6 +25,7 @@ namespace ozk {
 constexpr int SPLIT_ROWS = 32;               // rows of a CTA: one per lane
 constexpr int SPLIT_MAX_WARPS = 8;           // a warp takes one K-block (8 elements) at a time
 constexpr int SPLIT_MAX_KG = 8;              // CTAs of a cluster that share a row block's K-blocks
+constexpr int SPLIT_GMAX_KG = 16, SPLIT_GMAX_KB = 384;   // row maxima by a launch of their own: launch_split
 
 // Digits of 8 elements for a compile-time slice count SF <= 10 (nbits = 8 SF - 1; 64-bit images, 96-bit
 // ones for SF = 9 and 10), with no dependent chain per digit.  With C = 128 (1 + 256 + ... + 256^(SF-2)), Y = X + C holds
@@ -287,10 +288,11 @@ __device__ __forceinline__ unsigned long long block_max(const longlong2 (&v)[8])
 // Both operands of one emulated GEMM in one launch: blockIdx.z selects the side.  A CTA owns 32
 // rows, one per lane; warp w takes the K-blocks w, w + nwarps, ... of its share.  With kgroups > 1
 // the CTAs of a cluster share a row block's K-blocks and exchange their row maxima through
-// distributed shared memory.  A share of at most one K-block per warp is read from memory once and
-// kept in registers between the maximum and the digits; longer shares are read twice.  Non-finite
+// distributed shared memory; GIVEN: the row maxima are there already (gmax: split_rowmax_kernel) and
+// the CTAs, no cluster then, have nothing to exchange.  A share of at most one K-block per warp is read from memory once
+// and kept in registers between the maximum and the digits; longer shares are read twice.  Non-finite
 // scalars flag OZK_ERR_NONFINITE, make their row's exponent 0 and are split as zero.
-template <int SF, bool W64, int SIDE>
+template <int SF, bool W64, int SIDE, bool GIVEN>
 __device__ __forceinline__ void split_rows(const SplitParams& p, unsigned long long (&wmax)[SPLIT_MAX_WARPS][SPLIT_ROWS],
                                            unsigned long long (&cmax)[SPLIT_MAX_KG][SPLIT_ROWS]) {
   const int z = blockIdx.y;
@@ -301,7 +303,7 @@ __device__ __forceinline__ void split_rows(const SplitParams& p, unsigned long l
   const int rank = static_cast<int>(blockIdx.x) % kgs;
   const int r0 = (static_cast<int>(blockIdx.x) / kgs) * SPLIT_ROWS;
   if (r0 >= R) return;                                 // the same for every CTA of the cluster
-  if (kgs > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  if (!GIVEN && kgs > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   const longlong2* __restrict__ P = reinterpret_cast<const longlong2*>(single ? p.X1 + z * p.zstride1 : p.X[z]);
   const long long ld = single ? p.ld1 : p.ld[z];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -309,11 +311,13 @@ __device__ __forceinline__ void split_rows(const SplitParams& p, unsigned long l
   const bool rok = r < R;
   const int nkb = (K + 7) >> 3, share = (nkb + kgs - 1) / kgs;
   const int kb0 = rank * share, kb1 = min(nkb, kb0 + share);
-  const bool resident = share <= nw;
+  const bool resident = !GIVEN && share <= nw;
 
   longlong2 v[8];
   unsigned long long mx = 0ull;
-  if (rok) {
+  if (rok && GIVEN) {
+    mx = p.gmax[z * p.exp_stride + r];
+  } else if (rok) {
     if (resident) {
       if (kb0 + warp < kb1) {
         load_block(p, P, ld, r, 8 * (kb0 + warp), K, v);
@@ -326,10 +330,12 @@ __device__ __forceinline__ void split_rows(const SplitParams& p, unsigned long l
       }
     }
   }
-  wmax[warp][lane] = mx;
-  __syncthreads();
-  for (int w = 0; w < nw; ++w) mx = max(mx, wmax[w][lane]);
-  if (kgs > 1) {
+  if constexpr (!GIVEN) {
+    wmax[warp][lane] = mx;
+    __syncthreads();
+    for (int w = 0; w < nw; ++w) mx = max(mx, wmax[w][lane]);
+  }
+  if (!GIVEN && kgs > 1) {
     asm volatile("barrier.cluster.wait.aligned;" ::: "memory");      // every peer has started
     if (warp < kgs) {
       uint32_t dst;
@@ -384,14 +390,72 @@ __device__ __forceinline__ void split_rows(const SplitParams& p, unsigned long l
   }
 }
 
-template <int SF, bool W64>
+template <int SF, bool W64, bool GIVEN>
 __global__ void __launch_bounds__(SPLIT_MAX_WARPS * 32, 2) split_kernel(const __grid_constant__ SplitPair pp) {
   __shared__ unsigned long long wmax[SPLIT_MAX_WARPS][SPLIT_ROWS];     // row maxima of the warps
   __shared__ unsigned long long cmax[SPLIT_MAX_KG][SPLIT_ROWS];        // and of the cluster's CTAs
   grid_dependency_wait();
   launch_dependents();
-  if (pp.s[blockIdx.z].side == 0) split_rows<SF, W64, 0>(pp.s[blockIdx.z], wmax, cmax);
-  else split_rows<SF, W64, 1>(pp.s[blockIdx.z], wmax, cmax);
+  if (pp.s[blockIdx.z].side == 0) split_rows<SF, W64, 0, GIVEN>(pp.s[blockIdx.z], wmax, cmax);
+  else split_rows<SF, W64, 1, GIVEN>(pp.s[blockIdx.z], wmax, cmax);
+}
+
+// Row maxima ahead of the split: the same CTAs (kgroups per row block), each over its share of the
+// K-blocks; one 64-bit atomicMax per row and CTA into gmax, which the launcher clears.
+__global__ void __launch_bounds__(SPLIT_MAX_WARPS * 32, 2) split_rowmax_kernel(const __grid_constant__ SplitPair pp) {
+  __shared__ unsigned long long wmax[SPLIT_MAX_WARPS][SPLIT_ROWS];
+  grid_dependency_wait();
+  launch_dependents();
+  const SplitParams& p = pp.s[blockIdx.z];
+  const int z = blockIdx.y;
+  const bool single = p.X == nullptr;
+  const int R = single ? p.rows1 : p.rows[z];
+  const int K = single ? p.k1 : p.kdim[z];
+  const int rank = static_cast<int>(blockIdx.x) % p.kgroups;
+  const int r0 = (static_cast<int>(blockIdx.x) / p.kgroups) * SPLIT_ROWS;
+  if (r0 >= R) return;
+  const longlong2* __restrict__ P = reinterpret_cast<const longlong2*>(single ? p.X1 + z * p.zstride1 : p.X[z]);
+  const long long ld = single ? p.ld1 : p.ld[z];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int r = r0 + lane;
+  const int nkb = (K + 7) >> 3, share = (nkb + p.kgroups - 1) / p.kgroups;
+  const int kb0 = rank * share, kb1 = min(nkb, kb0 + share);
+  unsigned long long mx = 0ull;
+  if (r < R)
+    for (int kb = kb0 + warp; kb < kb1; kb += nw) {
+      longlong2 v[8];
+      load_block(p, P, ld, r, 8 * kb, K, v);
+      mx = max(mx, block_max(v));
+    }
+  wmax[warp][lane] = mx;
+  __syncthreads();
+  if (warp != 0 || r >= R) return;
+  for (int w = 1; w < nw; ++w) mx = max(mx, wmax[w][lane]);
+  if (mx) atomicMax(&p.gmax[z * p.exp_stride + r], mx);
+}
+
+// compile-time slice counts 3..10 (nbits = 8 S - 1 on every side); the test hook's digit copy and
+// other slice counts take the run-time form
+template <bool GIVEN>
+static void launch_instances(const cudaLaunchConfig_t& cfg, const SplitPair& pp) {
+  int sf = pp.s[0].S;
+  for (int sd = 0; sd < pp.nsides; ++sd)
+    if (pp.s[sd].S != sf || pp.s[sd].nbits != 8 * sf - 1 || pp.s[sd].dbg_digits) sf = 0;
+  switch (sf) {
+    case 3: cudaLaunchKernelEx(&cfg, split_kernel<3, true, GIVEN>, pp); break;
+    case 4: cudaLaunchKernelEx(&cfg, split_kernel<4, true, GIVEN>, pp); break;
+    case 5: cudaLaunchKernelEx(&cfg, split_kernel<5, true, GIVEN>, pp); break;
+    case 6: cudaLaunchKernelEx(&cfg, split_kernel<6, true, GIVEN>, pp); break;
+    case 7: cudaLaunchKernelEx(&cfg, split_kernel<7, true, GIVEN>, pp); break;
+    case 8: cudaLaunchKernelEx(&cfg, split_kernel<8, true, GIVEN>, pp); break;
+    case 9: cudaLaunchKernelEx(&cfg, split_kernel<9, false, GIVEN>, pp); break;
+    case 10: cudaLaunchKernelEx(&cfg, split_kernel<10, false, GIVEN>, pp); break;
+    default:
+      if (pp.s[0].nbits <= 62 && (pp.nsides < 2 || pp.s[1].nbits <= 62))
+        cudaLaunchKernelEx(&cfg, split_kernel<0, true, GIVEN>, pp);
+      else
+        cudaLaunchKernelEx(&cfg, split_kernel<0, false, GIVEN>, pp);
+  }
 }
 
 void launch_split(const SplitParams& a, int rows_a, const SplitParams* b, int rows_b, int kmax, int batch,
@@ -411,11 +475,24 @@ void launch_split(const SplitParams& a, int rows_a, const SplitParams* b, int ro
   while (kg < SPLIT_MAX_KG && ((nkb + kg - 1) / kg > SPLIT_MAX_WARPS ||
                                (ctas * kg < 2LL * gpu_sm_count() && nkb / (2 * kg) >= 8)))
     kg *= 2;
+  // Clusters of 8 over few row blocks leave most of a GPU idle that holds 2 CTAs an SM, and read a long
+  // share twice.  Where at least 16 CTAs a row block find room, the row maxima of 384 K-blocks (K = 3072)
+  // or more are taken by a launch of their own, and every row block's K-blocks are dealt to all those CTAs,
+  // at least 8 to each.  Products at S = 7 with clusters and so: 32 x 32 x 2048 51 and 44 us, x 4096 88 and
+  // 63, x 32768 578 and 318; 256 x 256 (19 CTAs a row block) x 1024 39 and 44, x 4096 105 and 94; at S = 5
+  // 16 x 16 x 2048 103 and 105, x 3072 148 and 145; 500 x 500 (9 CTAs a row block) x 4096 225 and 241.
+  const long long fill = std::min<long long>(2LL * gpu_sm_count() / std::max(1LL, ctas), nkb / SPLIT_MAX_WARPS);
+  const bool given = a.gmax && (!b || b->gmax) && fill >= SPLIT_GMAX_KG && nkb >= SPLIT_GMAX_KB;
+  if (given) kg = static_cast<int>(fill);
   const int share = (nkb + kg - 1) / kg;
-  for (int sd = 0; sd < pp.nsides; ++sd) pp.s[sd].kgroups = kg;
+  for (int sd = 0; sd < pp.nsides; ++sd) {
+    pp.s[sd].kgroups = kg;
+    if (!given) pp.s[sd].gmax = nullptr;
+    else cudaMemsetAsync(pp.s[sd].gmax, 0, sizeof(unsigned long long) * pp.s[sd].exp_stride * batch, st);
+  }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(rblocks * kg), static_cast<unsigned>(batch), static_cast<unsigned>(pp.nsides));
-  cfg.blockDim = dim3(32u * static_cast<unsigned>(std::max(std::min(share, SPLIT_MAX_WARPS), kg)));
+  cfg.blockDim = dim3(32u * static_cast<unsigned>(given ? SPLIT_MAX_WARPS : std::max(std::min(share, SPLIT_MAX_WARPS), kg)));
   cfg.stream = st;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -423,26 +500,15 @@ void launch_split(const SplitParams& a, int rows_a, const SplitParams* b, int ro
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   at[1] = pdl_attribute(st);
-  cfg.attrs = kg > 1 ? at : at + 1;
-  cfg.numAttrs = kg > 1 ? 2 : 1;
-  // compile-time slice counts 3..10 (nbits = 8 S - 1 on every side); the test hook's digit copy and
-  // other slice counts take the run-time form
-  int sf = pp.s[0].S;
-  for (int sd = 0; sd < pp.nsides; ++sd)
-    if (pp.s[sd].S != sf || pp.s[sd].nbits != 8 * sf - 1 || pp.s[sd].dbg_digits) sf = 0;
-  switch (sf) {
-    case 3: cudaLaunchKernelEx(&cfg, split_kernel<3, true>, pp); break;
-    case 4: cudaLaunchKernelEx(&cfg, split_kernel<4, true>, pp); break;
-    case 5: cudaLaunchKernelEx(&cfg, split_kernel<5, true>, pp); break;
-    case 6: cudaLaunchKernelEx(&cfg, split_kernel<6, true>, pp); break;
-    case 7: cudaLaunchKernelEx(&cfg, split_kernel<7, true>, pp); break;
-    case 8: cudaLaunchKernelEx(&cfg, split_kernel<8, true>, pp); break;
-    case 9: cudaLaunchKernelEx(&cfg, split_kernel<9, false>, pp); break;
-    case 10: cudaLaunchKernelEx(&cfg, split_kernel<10, false>, pp); break;
-    default:
-      if (pp.s[0].nbits <= 62 && (pp.nsides < 2 || pp.s[1].nbits <= 62)) cudaLaunchKernelEx(&cfg, split_kernel<0, true>, pp);
-      else cudaLaunchKernelEx(&cfg, split_kernel<0, false>, pp);
+  const bool cluster = kg > 1 && !given;
+  cfg.attrs = cluster ? at : at + 1;
+  cfg.numAttrs = cluster ? 2 : 1;
+  if (given) {
+    cudaLaunchKernelEx(&cfg, split_rowmax_kernel, pp);
+    record_launch();
   }
+  if (given) launch_instances<true>(cfg, pp);
+  else launch_instances<false>(cfg, pp);
   record_launch();
 }
 
