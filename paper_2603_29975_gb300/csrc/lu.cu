@@ -16,13 +16,20 @@
 namespace ozk {
 
 constexpr int GJ_THREADS = 256;
+constexpr int GJ_MAX_NB = 64;                // order of the blocks and right-hand sides of gj_solve_kernel
 
-
+// Raises the dynamic shared memory that launches of a kernel may ask for to `most`, the largest of any
+// launch: the limit is the kernel's, so it is set to the same value by every call, and a thread whose
+// launch needs less cannot lower it between another's setting and launch.
+template <typename K>
+static void allow_smem(K kernel, size_t most) {
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most));
+}
 
 __global__ void __launch_bounds__(GJ_THREADS)
 gj_solve_kernel(const GjParams p) {
   extern __shared__ double2 A[];            // [nb][w] row-major, w = nb + nrhs
-  __shared__ double2 fcol[64];
+  __shared__ double2 fcol[GJ_MAX_NB];
   __shared__ int s_piv;
   __shared__ double s_pval;
   const int z = blockIdx.x;
@@ -788,8 +795,7 @@ lu_panel_kernel(double2* D, long long ldd, int w, double2* Rs, long long ldr, in
 void launch_lu_panel(double2* D, long long ldd, int w, double2* Rs, long long ldr, int ncols, int* status,
                      cudaStream_t st) {
   const size_t smem = sizeof(double2) * static_cast<size_t>(w) * w;
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(lu_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  allow_smem(lu_panel_kernel, sizeof(double2) * GJINV_MAX * GJINV_MAX);
   lu_panel_kernel<<<1, GJINV_THREADS, smem, st>>>(D, ldd, w, Rs, ldr, ncols, status);
   record_launch();
 }
@@ -864,9 +870,11 @@ void launch_gjinv(const GjParams& p, int max_w, int batch, cudaStream_t st) {
   const bool two = 2 * batch <= sms || (batch <= sms && max_w <= 80);
   const int C = 8 * batch <= sms ? 8 : (4 * batch <= sms ? 4 : (two ? 2 : 1));
   if (C > 1) {
-    const size_t smem = sizeof(double2) * (static_cast<size_t>((max_w + C - 1) / C) * max_w +
-                                           static_cast<size_t>(GJC_SLOTS) * (max_w + 2));
-    cudaFuncSetAttribute(gjinv_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    auto bytes = [](int w, int ctas) {
+      return sizeof(double2) * (static_cast<size_t>((w + ctas - 1) / ctas) * w + static_cast<size_t>(GJC_SLOTS) * (w + 2));
+    };
+    const size_t smem = bytes(max_w, C);
+    allow_smem(gjinv_cluster_kernel, bytes(GJINV_MAX, 2));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(static_cast<unsigned>(batch * C));
     cfg.blockDim = dim3(GJC_THREADS);
@@ -892,8 +900,7 @@ void launch_gjinv(const GjParams& p, int max_w, int batch, cudaStream_t st) {
     if (single) return;
   }
   const size_t smem = sizeof(double2) * static_cast<size_t>(max_w) * max_w;
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(gjinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  allow_smem(gjinv_kernel, sizeof(double2) * GJINV_MAX * GJINV_MAX);
   gjinv_kernel<<<batch, GJINV_THREADS, smem, st>>>(p, reg ? GJR_MIN_W : 0, reg ? GJR_W : 0);
   record_launch();
 }
@@ -903,7 +910,7 @@ void launch_gj(const GjParams& p, int max_nb, int max_nrhs, int batch, cudaStrea
     gj16_kernel<<<batch, GJ16_THREADS, 0, st>>>(p);
   } else {
     const size_t smem = sizeof(double2) * static_cast<size_t>(max_nb) * (max_nb + max_nrhs);
-    if (smem > 48 * 1024) cudaFuncSetAttribute(gj_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    allow_smem(gj_solve_kernel, sizeof(double2) * GJ_MAX_NB * 2 * GJ_MAX_NB);
     gj_solve_kernel<<<batch, GJ_THREADS, smem, st>>>(p);
   }
   record_launch();

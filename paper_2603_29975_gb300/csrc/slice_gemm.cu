@@ -16,7 +16,7 @@ static size_t gemm_smem_bytes(int S, int BN, int nstage) {
 
 int gemm_stages(int S, int BN) {
   int n = 6;
-  while (n > 0 && gemm_smem_bytes(S, BN, n) > 227 * 1024) --n;
+  while (n > 0 && gemm_smem_bytes(S, BN, n) > GEMM_SMEM_MAX) --n;
   return n;
 }
 

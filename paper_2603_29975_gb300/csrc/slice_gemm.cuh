@@ -41,7 +41,7 @@ constexpr int GEMM_EPI_WARPS = 16;
 constexpr int GEMM_CTRL_WARPS = 4;
 constexpr int GEMM_THREADS = (GEMM_CTRL_WARPS + GEMM_EPI_WARPS) * 32;
 constexpr int GEMM_CTRL_REGS = 64, GEMM_EPI_REGS = 104;
-
+constexpr int GEMM_SMEM_MAX = 227 * 1024;        // shared memory of a CTA (all of it dynamic)
 
 // Exact sums at the ends of the binary64 exponent range, one rounding in 128 bits.
 static __device__ __noinline__ double round_far(long long H, long long L, int s8, int E) {
@@ -1178,8 +1178,9 @@ slice_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 template <int BN, int SF, bool KS>
 inline void launch_instance(const CUtensorMap& ta, const CUtensorMap& tb, const GemmParams& p, int grid, size_t smem,
                             cudaStream_t st) {
-  cudaFuncSetAttribute(slice_gemm_kernel<BN, SF, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       static_cast<int>(smem));
+  // the limit is the kernel's, not the launch's: the same value from every call, so that a thread whose
+  // launch needs less cannot lower it between another's setting and launch
+  cudaFuncSetAttribute(slice_gemm_kernel<BN, SF, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM_MAX);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(grid));
   cfg.blockDim = dim3(GEMM_THREADS);
