@@ -595,22 +595,25 @@ gjinv_cluster_kernel(const GjParams p, int C, int max_w) {
   };
 
   if (rank == 0 && tid < wp) search(0, tid < w ? A[tid] : make_double2(0.0, 0.0), A);
-  bool singular = false, quit = false;
+  // waits for step k's message; false when the limit ran out
+  auto received = [&](int k) {
+    const uint32_t parity = static_cast<uint32_t>(k / GJC_SLOTS) & 1u;
+    const long long t0 = clock64();
+    while (!mbar_try_wait(&bar[k % GJC_SLOTS], parity))
+      if (clock64() - t0 > kWaitBudget) return false;
+    return true;
+  };
+  bool singular = false;
+  int left = w;                                             // the step at which this CTA gave up, if it did
   for (int k = 0; k < w; ++k) {
     if (k > 0 && k % (GJC_SLOTS / 2) == 0) cluster_sync();  // every CTA is done with the steps below k
-    if (quit) continue;                                     // (only the cluster's barriers are kept)
     const int slot = k % GJC_SLOTS;
     const double2* msg = ring + static_cast<size_t>(slot) * pitch;
     const bool mine = static_cast<unsigned>(k - c0) < static_cast<unsigned>(ncol);
-    if (!mine) {
-      const uint32_t parity = static_cast<uint32_t>(k / GJC_SLOTS) & 1u;
-      const long long t0 = clock64();
-      while (!mbar_try_wait(&bar[slot], parity))
-        if (clock64() - t0 > kWaitBudget) { *static_cast<volatile int*>(&gave_up) = k + 1; break; }
-    }
+    if (!mine && !received(k)) *static_cast<volatile int*>(&gave_up) = k + 1;
     __syncthreads();                                        // message k is here, the updates of step k - 1 are done
     // a step's failed wait is seen by every thread after that step's barrier
-    if (!mine && *static_cast<volatile int*>(&gave_up) == k + 1) { quit = true; continue; }
+    if (!mine && *static_cast<volatile int*>(&gave_up) == k + 1) { left = k; break; }
     // the chain goes on in this CTA
     const bool ahead = static_cast<unsigned>(k + 1 - c0) < static_cast<unsigned>(ncol);
     const int jn = k + 1 - c0;                              // its column's local index
@@ -687,14 +690,26 @@ gjinv_cluster_kernel(const GjParams p, int C, int max_w) {
       }
     }
   }
+  // a CTA that gave up keeps the cluster's barriers, and its last thread receives what the others still
+  // send: no copy into this CTA may be in flight when it ends.  After a message that does not come (this
+  // CTA's own, or one of another that gave up) none can follow.
+  bool more = true;
+  for (int k = left; k < w; ++k) {
+    if (k > left && k % (GJC_SLOTS / 2) == 0) cluster_sync();
+    if (tid == GJC_THREADS - 1 && more) {
+      more = k / nc != rank && received(k);
+      if (more && k + GJC_SLOTS < w) arm(k + GJC_SLOTS);
+    }
+    __syncwarp();
+  }
   __syncthreads();
   if (tid == 0 && gave_up) flag_error(p.status, OZK_ERR_TIMEOUT);
   if (singular && tid == 0 && rank == 0) flag_error(p.status, OZK_ERR_SINGULAR);
   for (int jl = cg; jl < ncol; jl += ng)
     if (r < w) X[r + static_cast<long long>(dst[c0 + jl]) * ldx] =
         singular ? make_double2(0.0, 0.0) : A[static_cast<size_t>(jl) * max_w + r];
-  // no CTA leaves while another may still send to it (every message is received before its step, but
-  // a singular or abandoned block ends early)
+  // no CTA leaves while another may still send to it or has yet to receive from it (a singular block ends
+  // early; a CTA that gave up has received what was sent)
   cluster_sync();
 }
 
