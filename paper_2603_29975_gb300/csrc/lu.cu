@@ -234,13 +234,12 @@ gjinv_kernel(const GjParams p, int skip_lo, int skip_hi) {
   __shared__ int s_piv, s_sing;
   __shared__ double2 s_pinv;
   const int z = blockIdx.x;
-  const bool single = p.D == nullptr;
-  const int w = single ? p.nb1 : p.nb[z];
+  const int w = p.nb[z];
   if (w <= 0 || (w > skip_lo && w <= skip_hi)) return;  // those blocks: gjinv_reg_kernel
-  const double2* D = single ? p.D1 : p.D[z];
-  const long long ldd = single ? p.ldd1 : p.ldd[z];
-  double2* X = single ? p.X1 : p.X[z];
-  const long long ldx = single ? p.ldx1 : p.ldx[z];
+  const double2* D = p.D[z];
+  const long long ldd = p.ldd[z];
+  double2* X = p.X[z];
+  const long long ldx = p.ldx[z];
   const int tid = threadIdx.x;
   const int ww = w * w;
   for (int idx = tid; idx < ww; idx += GJINV_THREADS) {
@@ -369,13 +368,12 @@ gjinv_reg_kernel(const GjParams p) {
   __shared__ int s_piv, s_sing;
   __shared__ double2 s_pinv;
   const int z = blockIdx.x;
-  const bool single = p.D == nullptr;
-  const int w = single ? p.nb1 : p.nb[z];
+  const int w = p.nb[z];
   if (w <= GJR_MIN_W || w > GJR_W) return;             // gjinv_kernel's blocks
-  const double2* D = single ? p.D1 : p.D[z];
-  const long long ldd = single ? p.ldd1 : p.ldd[z];
-  double2* X = single ? p.X1 : p.X[z];
-  const long long ldx = single ? p.ldx1 : p.ldx[z];
+  const double2* D = p.D[z];
+  const long long ldd = p.ldd[z];
+  double2* X = p.X[z];
+  const long long ldx = p.ldx[z];
   const int tid = threadIdx.x;
   const int j = tid & (GJR_W - 1), rb = tid / GJR_W;
   double2 a[GJR_RPT];
@@ -882,7 +880,7 @@ void launch_gjinv(const GjParams& p, int max_w, int batch, cudaStream_t st) {
   // inverts a block depends on its own order and on whether the launch has at most one block per SM
   // only, so a block comes out the same alone and in a batch of that size.
   const int sms = gpu_sm_count();
-  const bool two = 2 * batch <= sms || (batch <= sms && max_w <= 80);
+  const bool two = batch == 1 || 2 * batch <= sms || (batch <= sms && max_w <= 80);
   const int C = 8 * batch <= sms ? 8 : (4 * batch <= sms ? 4 : (two ? 2 : 1));
   if (C > 1) {
     auto bytes = [](int w, int ctas) {
@@ -907,12 +905,11 @@ void launch_gjinv(const GjParams& p, int max_w, int batch, cudaStream_t st) {
     record_launch();
     return;
   }
-  const bool single = p.D == nullptr;                      // one block, of order max_w
-  const bool reg = max_w > GJR_MIN_W && batch <= sms && (!single || max_w <= GJR_W);
+  // (a single block, whose pointers come without tables, has always taken a cluster)
+  const bool reg = batch <= sms;                           // a block above order 80 is among them
   if (reg) {
     gjinv_reg_kernel<<<batch, GJR_THREADS, 0, st>>>(p);
     record_launch();
-    if (single) return;
   }
   const size_t smem = sizeof(double2) * static_cast<size_t>(max_w) * max_w;
   allow_smem(gjinv_kernel, sizeof(double2) * GJINV_MAX * GJINV_MAX);
