@@ -277,9 +277,33 @@ struct EmuGemm {
   cudaStream_t stream = nullptr;
 };
 
+// pairs of each weight class g = s + t of the pair set (np[0..G))
+static void group_pairs(int S, int pair_mode, int (&np)[32]) {
+  for (int& v : np) v = 0;
+  for (int s = 1; s <= S; ++s)
+    for (int t = 1; t <= S; ++t) {
+      if (pair_mode == PAIRS_DIAG ? s != t : (pair_mode != OZK_PAIRS_FULL && s + t > S + 1)) continue;
+      const int gi = pair_mode == PAIRS_DIAG ? s - 1 : s + t - 2;
+      if (gi < 32) ++np[gi];
+    }
+}
+// Whether four groups' sums over the whole K, combined with their weights, stay below 2^63 in magnitude
+// (0.99 of it, so that the next four's carry fits too): the epilogues keep every quad [4 q, 4 q + 4) of
+// the groups in 64 bits.  Digit products are at most 2^14; triangular sets reach the limit at K of about
+// 3.3 million for S = 8..10 (groups 4..7: 5 pairs at the quad's top) and 16 million for S = 4..7.
+static bool quads_fit64(int G, const int (&np)[32], long long kterms) {
+  for (int q = 0; q < G; q += 4) {
+    double b = 0.0;
+    for (int g = q; g < std::min(q + 4, G); ++g) b = 256.0 * b + np[g];
+    if (b * 16384.0 * static_cast<double>(kterms) >= 0.99 * 0x1.0p63) return false;
+  }
+  return true;
+}
+
 struct GemmPlan {
   int G, BN, maxpairs, npairs, kpad, rowsA, rowsB, chunk_kb, kblocks, magic;
   int ksplit;                                 // split-K units per tile (single problems with few tiles)
+  int wide;                                   // the sums of four groups may pass 64 bits (very long K)
   size_t offA, offB, offE, offF, offT, offP, offGA, offGB, total;
 };
 
@@ -327,13 +351,16 @@ ozk_status_t plan_gemm(const EmuGemm& g, GemmPlan* P) {
   // general modes)
   P->ksplit = 1;
   P->offP = off;
+  int np[32];
+  group_pairs(S, g.pair_mode, np);
+  P->wide = quads_fit64(P->G, np, 16LL * P->kblocks) ? 0 : 1;
   {
     const double terms = 16.0 * P->kblocks * P->maxpairs;
     const int bits = static_cast<int>(std::ceil(std::log2(terms))) + 14 + 8 * (P->G - 1) + 1;
     const bool fit64 = P->G <= 5 && bits <= 63;
     const bool modes = g.mode < 0 || g.mode == EPI_STORE || g.mode == EPI_LU || g.mode == EPI_GENERAL;
     if (g.ksplit_ok && g.batch == 1 && g.tm == nullptr && !g.remap && !g.crow && !diag && g.pair_mode == OZK_PAIRS_TRI &&
-        P->BN == 64 && P->G <= 8 && !fit64 && modes && g.m > 0 && g.n > 0) {
+        P->BN == 64 && P->G <= 8 && !fit64 && !P->wide && modes && g.m > 0 && g.n > 0) {
       const int nch = (P->kblocks + P->chunk_kb - 1) / P->chunk_kb;
       const long long tiles = static_cast<long long>((g.m + 127) / 128) * ((2LL * g.n + 63) / 64);
       const int sms = gpu_sm_count();
@@ -414,14 +441,8 @@ ozk_status_t run_emulated(ozk_context* h, const EmuGemm& g, size_t ws_offset = 0
   {
     // group g receives the products of its own pairs only: 16 per K-block and pair, each at most
     // 2^14 in magnitude, so a group of np pairs stays within 2^22 when 16 np chunk_kb <= 256
-    int np[32] = {0};
-    for (int s1 = 1; s1 <= S; ++s1)
-      for (int t1 = 1; t1 <= S; ++t1) {
-        if (diag && s1 != t1) continue;
-        if (!diag && g.pair_mode != OZK_PAIRS_FULL && s1 + t1 > S + 1) continue;
-        const int gi = diag ? s1 - 1 : s1 + t1 - 2;
-        if (gi < 32) ++np[gi];
-      }
+    int np[32];
+    group_pairs(S, g.pair_mode, np);
     gp.magic_mask = 0;
     for (int gi = 0; gi < std::min(P.G, 32); ++gi)
       if (np[gi] > 0 && 16LL * np[gi] * P.chunk_kb <= 256) gp.magic_mask |= static_cast<int>(1u << gi);
@@ -432,6 +453,7 @@ ozk_status_t run_emulated(ozk_context* h, const EmuGemm& g, size_t ws_offset = 0
     const double terms = 16.0 * P.kblocks * P.maxpairs;
     const int bits = static_cast<int>(std::ceil(std::log2(terms))) + 14 + 8 * (P.G - 1) + 1;
     gp.fit64 = (P.G <= 5 && bits <= 63) ? 1 : 0;
+    gp.wide = P.wide && !gp.fit64 ? 1 : 0;
   }
   gp.fullset = g.pair_mode == OZK_PAIRS_FULL ? 1 : 0;
   const int gmax = (g.pair_mode == OZK_PAIRS_FULL) ? 2 * S : S + 1;

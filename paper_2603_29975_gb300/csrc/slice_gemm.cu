@@ -44,8 +44,8 @@ void launch_slice_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const GemmP
   const long long ntiles = static_cast<long long>(p.tpp) * batch * std::max(1, p.ksplit);
   const int grid = static_cast<int>(std::min<long long>(ntiles, num_sms()));
   const size_t smem = gemm_smem_bytes(p.S, BN, p.nstage);
-  // the compile-time instances hold only the fast epilogues (no integer group dumps)
-  const bool tri = !p.fullset && !p.diag_pairs && p.mode != EPI_GROUPS && p.mode != EPI_RESIDUES;
+  // the compile-time instances hold only the fast epilogues (no integer group dumps, sums in 64 bits)
+  const bool tri = !p.fullset && !p.diag_pairs && !p.wide && p.mode != EPI_GROUPS && p.mode != EPI_RESIDUES;
   const bool ks = p.ksplit > 1;
   // 23 to 63 bits (S = 3..8): compact instances of one schedule and epilogue each; split K only for
   // S = 7, the precision of the batched contour workload (its unit bookkeeping costs the others
