@@ -511,6 +511,27 @@ __device__ __forceinline__ void named_sync(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
+// Step k of a CTA that gave up: it keeps the cluster's barriers, and its last thread receives what the
+// others still send: no copy into this CTA may be in flight when it ends.  After a message that does not
+// come (this CTA's own, or one of another that gave up) none can follow, and gave_up turns negative.  A
+// function of its own, so that the step loop keeps its code (inlined: order 112 345 instead of 334 us).
+static __device__ __noinline__ void gjc_drain(uint64_t* bar, int k, int w, int nc, int rank, uint32_t msg_bytes,
+                                                   volatile int* gave_up) {
+  if (threadIdx.x == GJC_THREADS - 1 && *gave_up > 0) {
+    uint64_t* b = &bar[k % GJC_SLOTS];
+    const uint32_t parity = static_cast<uint32_t>(k / GJC_SLOTS) & 1u;
+    const long long t0 = clock64();
+    bool came = k / nc != rank;
+    while (came && !mbar_try_wait(b, parity)) came = clock64() - t0 <= kWaitBudget;
+    if (!came) *gave_up = -1;
+    else if (k + GJC_SLOTS < w) {
+      if ((k + GJC_SLOTS) / nc == rank) mbar_arrive(b);
+      else mbar_arrive_expect_tx(b, msg_bytes);
+    }
+  }
+  __syncwarp();
+}
+
 __global__ void __launch_bounds__(GJC_THREADS)
 gjinv_cluster_kernel(const GjParams p, int C, int max_w) {
   extern __shared__ double2 dyn[];          // [columns of this CTA][max_w], then the ring [GJC_SLOTS][max_w + 2]
@@ -593,25 +614,27 @@ gjinv_cluster_kernel(const GjParams p, int C, int max_w) {
   };
 
   if (rank == 0 && tid < wp) search(0, tid < w ? A[tid] : make_double2(0.0, 0.0), A);
-  // waits for step k's message; false when the limit ran out
-  auto received = [&](int k) {
-    const uint32_t parity = static_cast<uint32_t>(k / GJC_SLOTS) & 1u;
-    const long long t0 = clock64();
-    while (!mbar_try_wait(&bar[k % GJC_SLOTS], parity))
-      if (clock64() - t0 > kWaitBudget) return false;
-    return true;
-  };
-  bool singular = false;
-  int left = w;                                             // the step at which this CTA gave up, if it did
+  bool singular = false, quit = false;
   for (int k = 0; k < w; ++k) {
     if (k > 0 && k % (GJC_SLOTS / 2) == 0) cluster_sync();  // every CTA is done with the steps below k
+    if (quit) { gjc_drain(bar, k, w, nc, rank, msg_bytes, &gave_up); continue; }
     const int slot = k % GJC_SLOTS;
     const double2* msg = ring + static_cast<size_t>(slot) * pitch;
     const bool mine = static_cast<unsigned>(k - c0) < static_cast<unsigned>(ncol);
-    if (!mine && !received(k)) *static_cast<volatile int*>(&gave_up) = k + 1;
+    if (!mine) {
+      const uint32_t parity = static_cast<uint32_t>(k / GJC_SLOTS) & 1u;
+      const long long t0 = clock64();
+      while (!mbar_try_wait(&bar[slot], parity))
+        if (clock64() - t0 > kWaitBudget) { *static_cast<volatile int*>(&gave_up) = k + 1; break; }
+    }
     __syncthreads();                                        // message k is here, the updates of step k - 1 are done
     // a step's failed wait is seen by every thread after that step's barrier
-    if (!mine && *static_cast<volatile int*>(&gave_up) == k + 1) { left = k; break; }
+    if (!mine && *static_cast<volatile int*>(&gave_up) == k + 1) {
+      quit = true;
+      __syncthreads();                                      // every thread has read gave_up
+      gjc_drain(bar, k, w, nc, rank, msg_bytes, &gave_up);
+      continue;
+    }
     // the chain goes on in this CTA
     const bool ahead = static_cast<unsigned>(k + 1 - c0) < static_cast<unsigned>(ncol);
     const int jn = k + 1 - c0;                              // its column's local index
@@ -687,18 +710,6 @@ gjinv_cluster_kernel(const GjParams p, int C, int max_w) {
         *e = r == k ? x : y;
       }
     }
-  }
-  // a CTA that gave up keeps the cluster's barriers, and its last thread receives what the others still
-  // send: no copy into this CTA may be in flight when it ends.  After a message that does not come (this
-  // CTA's own, or one of another that gave up) none can follow.
-  bool more = true;
-  for (int k = left; k < w; ++k) {
-    if (k > left && k % (GJC_SLOTS / 2) == 0) cluster_sync();
-    if (tid == GJC_THREADS - 1 && more) {
-      more = k / nc != rank && received(k);
-      if (more && k + GJC_SLOTS < w) arm(k + GJC_SLOTS);
-    }
-    __syncwarp();
   }
   __syncthreads();
   if (tid == 0 && gave_up) flag_error(p.status, OZK_ERR_TIMEOUT);
