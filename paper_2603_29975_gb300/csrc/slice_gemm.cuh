@@ -1042,7 +1042,7 @@ slice_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       const int rl = quad * 32 + lane;           // row in the tile
       const int unch = (ti->kb1 - ti->kb0 + p.chunk_kb - 1) / p.chunk_kb;    // exactness chunks of this unit
       if constexpr (COLS == 16) {
-        if (SF > 0 || (G <= 8 && !p.wide && p.mode != EPI_GROUPS && p.mode != EPI_RESIDUES)) {
+        if (G <= 8 && (SF > 0 || !p.wide) && p.mode != EPI_GROUPS && p.mode != EPI_RESIDUES) {
           EpiCtx x;
           const RowInfo o = ti->row[rl];
           x.row = ti->row0 + rl; x.n2 = ti->n2; x.n0 = ti->n0; x.c0 = c0; x.tbase = tbase; x.sp = ti->sp;
