@@ -511,27 +511,6 @@ __device__ __forceinline__ void named_sync(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
-// Step k of a CTA that gave up: it keeps the cluster's barriers, and its last thread receives what the
-// others still send: no copy into this CTA may be in flight when it ends.  After a message that does not
-// come (this CTA's own, or one of another that gave up) none can follow, and gave_up turns negative.  A
-// function of its own, so that the step loop keeps its code (inlined: order 112 345 instead of 334 us).
-static __device__ __noinline__ void gjc_drain(uint64_t* bar, int k, int w, int nc, int rank, uint32_t msg_bytes,
-                                                   volatile int* gave_up) {
-  if (threadIdx.x == GJC_THREADS - 1 && *gave_up > 0) {
-    uint64_t* b = &bar[k % GJC_SLOTS];
-    const uint32_t parity = static_cast<uint32_t>(k / GJC_SLOTS) & 1u;
-    const long long t0 = clock64();
-    bool came = k / nc != rank;
-    while (came && !mbar_try_wait(b, parity)) came = clock64() - t0 <= kWaitBudget;
-    if (!came) *gave_up = -1;
-    else if (k + GJC_SLOTS < w) {
-      if ((k + GJC_SLOTS) / nc == rank) mbar_arrive(b);
-      else mbar_arrive_expect_tx(b, msg_bytes);
-    }
-  }
-  __syncwarp();
-}
-
 __global__ void __launch_bounds__(GJC_THREADS)
 gjinv_cluster_kernel(const GjParams p, int C, int max_w) {
   extern __shared__ double2 dyn[];          // [columns of this CTA][max_w], then the ring [GJC_SLOTS][max_w + 2]
@@ -617,7 +596,7 @@ gjinv_cluster_kernel(const GjParams p, int C, int max_w) {
   bool singular = false, quit = false;
   for (int k = 0; k < w; ++k) {
     if (k > 0 && k % (GJC_SLOTS / 2) == 0) cluster_sync();  // every CTA is done with the steps below k
-    if (quit) { gjc_drain(bar, k, w, nc, rank, msg_bytes, &gave_up); continue; }
+    if (quit) continue;                                     // (only the cluster's barriers are kept)
     const int slot = k % GJC_SLOTS;
     const double2* msg = ring + static_cast<size_t>(slot) * pitch;
     const bool mine = static_cast<unsigned>(k - c0) < static_cast<unsigned>(ncol);
@@ -629,12 +608,7 @@ gjinv_cluster_kernel(const GjParams p, int C, int max_w) {
     }
     __syncthreads();                                        // message k is here, the updates of step k - 1 are done
     // a step's failed wait is seen by every thread after that step's barrier
-    if (!mine && *static_cast<volatile int*>(&gave_up) == k + 1) {
-      quit = true;
-      __syncthreads();                                      // every thread has read gave_up
-      gjc_drain(bar, k, w, nc, rank, msg_bytes, &gave_up);
-      continue;
-    }
+    if (!mine && *static_cast<volatile int*>(&gave_up) == k + 1) { quit = true; continue; }
     // the chain goes on in this CTA
     const bool ahead = static_cast<unsigned>(k + 1 - c0) < static_cast<unsigned>(ncol);
     const int jn = k + 1 - c0;                              // its column's local index
@@ -649,7 +623,7 @@ gjinv_cluster_kernel(const GjParams p, int C, int max_w) {
         bulk_to_cta(mapa_u32(smem_u32(msg), c), smem_u32(msg), msg_bytes, mapa_u32(smem_u32(&bar[slot]), c));
       }
     }
-    if (sing) { singular = true; break; }
+    if (sing) { singular = true; wrow[0] = k; break; }      // (no search follows)
     if (chain) {
       double2 v = make_double2(0.0, 0.0);
       double2* col = A + static_cast<size_t>(jn) * max_w;
@@ -712,13 +686,30 @@ gjinv_cluster_kernel(const GjParams p, int C, int max_w) {
     }
   }
   __syncthreads();
-  if (tid == 0 && gave_up) flag_error(p.status, OZK_ERR_TIMEOUT);
+  if (singular) {                                           // the cluster's barriers of the steps left out
+#pragma unroll 1
+    for (int q = (wrow[0] / (GJC_SLOTS / 2) + 1) * (GJC_SLOTS / 2); q < w; q += GJC_SLOTS / 2) cluster_sync();
+  }
+  if (tid == 0 && gave_up) {
+    flag_error(p.status, OZK_ERR_TIMEOUT);
+    // what the others sent since is received, in order: no copy into this CTA may be in flight when it
+    // ends.  After a message that does not come (this CTA's own, or one of another that gave up) none can
+    // follow.
+    bool came = true;
+    for (int k = gave_up - 1; k < w && came; ++k) {
+      const long long t0 = clock64();
+      came = k / nc != rank;
+      while (came && !mbar_try_wait(&bar[k % GJC_SLOTS], static_cast<uint32_t>(k / GJC_SLOTS) & 1u))
+        came = clock64() - t0 <= kWaitBudget;
+      if (came && k + GJC_SLOTS < w) arm(k + GJC_SLOTS);
+    }
+  }
   if (singular && tid == 0 && rank == 0) flag_error(p.status, OZK_ERR_SINGULAR);
   for (int jl = cg; jl < ncol; jl += ng)
     if (r < w) X[r + static_cast<long long>(dst[c0 + jl]) * ldx] =
         singular ? make_double2(0.0, 0.0) : A[static_cast<size_t>(jl) * max_w + r];
-  // no CTA leaves while another may still send to it or has yet to receive from it (a singular block ends
-  // early; a CTA that gave up has received what was sent)
+  // no CTA leaves while another may still send to it or has yet to receive from it: singular or abandoned,
+  // every CTA has passed the same barriers, and one that gave up has received what was sent
   cluster_sync();
 }
 
