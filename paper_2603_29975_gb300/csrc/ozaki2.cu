@@ -26,6 +26,9 @@ __device__ __forceinline__ int sym_mod(int v, int m) {
   return 2 * r > m ? r - m : r;
 }
 
+// Residue planes in the slice split's layout, so that the same GEMM reads them: whole products (both splits,
+// GEMM, reconstruction) with rows of K-contiguous residues and so: 512^3, 16 moduli 1137 and 702 us, 6 moduli
+// 493 and 339; 2048^3, 16 moduli 14.7 and 8.8 ms; 1536 x 1536 x 192, 10 moduli 1213 and 926 us.
 __global__ void __launch_bounds__(RS_THREADS) residue_split_kernel(const SplitParams p, const Oz2Tables T) {
   const int z = blockIdx.y;
   const bool single = p.X == nullptr;

@@ -139,7 +139,9 @@ void launch_tile_prefix(const GemmParams& p, int BN, int batch, int* out, cudaSt
 void launch_finish_split(const GemmParams& p, cudaStream_t st);
 int gpu_sm_count();
 // not in a captured launch: replayed from a graph, the 256-solve step took 149.8 ms with such edges and
-// 143.6 without (its branches: pivot inverses beside the side stream's splits)
+// 143.2 without (its branches: pivot inverses beside the side stream's splits).  That graph alone was
+// measured with them; a captured single product does without what they give eager launches (64^3 at
+// S = 7: 24.6 us replayed, 20 eager)
 inline cudaLaunchAttribute pdl_attribute(cudaStream_t st) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   const bool known = cudaStreamIsCapturing(st, &cap) == cudaSuccess;

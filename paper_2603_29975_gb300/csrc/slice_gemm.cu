@@ -47,9 +47,9 @@ void launch_slice_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const GemmP
   // the compile-time instances hold only the fast epilogues (no integer group dumps, sums in 64 bits)
   const bool tri = !p.fullset && !p.diag_pairs && !p.wide && p.mode != EPI_GROUPS && p.mode != EPI_RESIDUES;
   const bool ks = p.ksplit > 1;
-  // 23 to 63 bits (S = 3..8): compact instances of one schedule and epilogue each; split K only for
-  // S = 7, the precision of the batched contour workload (its unit bookkeeping costs the others
-  // registers)
+  // 23 to 63 bits (S = 3..8): compact instances of one schedule and epilogue each.  Split K has an
+  // instance of its own at S = 7 only, the precision of the accuracy study's products; at S = 3..6 and 8
+  // it takes the run-time instance, which was not compared with more instances
   if (tri && BN == 32 && (p.S == 9 || p.S == 10)) {
     launch_slice_gemm_s910(ta, tb, p, grid, smem, st);
   } else if (tri && BN == 64 && p.S >= 3 && p.S <= 8 && (!ks || p.S == 7)) {

@@ -17,12 +17,14 @@
 //   * warp 2 finds the CTA's tiles ahead of the others and leaves them in a ring;
 //   * warps 4..19 drain the accumulators.  Every product of two digits is an integer of
 //     magnitude <= 2^14 and each accumulator receives at most 1024 of them per "exactness
-//     chunk" of K, so every FP32 value is an exact integer <= 2^24.  The epilogue converts
-//     it to int32 and adds it, shifted by its group weight 8 (g_max - g) bits, into a 64-bit
-//     (when the exact sum fits) or 128-bit integer per output element; after the last chunk
-//     that integer times 2^(e_i + f_j + c) is rounded once to binary64 (the int64 -> binary64
-//     conversion of the exact sum, or of a sticky-jammed 64-bit image of the 128-bit sum),
-//     then stored (C = Z), or subtracted from C (LU update), or combined with alpha/beta.
+//     chunk" of K, so every FP32 value is an exact integer <= 2^24.  The epilogue brings it into
+//     the low bits of a 32-bit word by one FP32 addition and adds groups in pairs, each with its
+//     weight of 8 (g_max - g) bits, into 64-bit integers: one per output element when the exact
+//     sum fits, else one per run of four groups (128-bit sums in the run-time schedules of many
+//     groups or a very long K).  After the last chunk their exact sum times 2^(e_i + f_j + c) is
+//     rounded once to binary64 (the int64 -> binary64 conversion of a 64-bit sum, integer
+//     operations on three 32-bit words or 128 bits otherwise), then stored (C = Z), or subtracted
+//     from C (LU update), or combined with alpha/beta.
 // No floating-point instruction touches the products' sums before that one rounding; the
 // only binary64 arithmetic after it is the subtraction / alpha-beta combination per element.
 #pragma once
@@ -49,7 +51,8 @@ static __device__ __noinline__ double round_far(long long H, long long L, int s8
 }
 
 // RN-even of (H 2^S8 + L) 2^E for int64 H, L and E such that every nonzero result is a normal number
-// (|H| < 2^56 and |L| < 2^(S8 + 30), S8 <= 32; S8 = 0: |H| < 2^63, no L).
+// (S8 <= 32; H + L 2^-S8 stays below 2^63 in magnitude, as the plan of the product checks by bounding H
+// and L by 0.99 2^63; S8 = 0: |H| < 2^63, no L).
 //   S8 = 0: the int64 -> binary64 conversion is that rounding, and the scaling an addition to the
 // exponent field.
 //   S8 > 0: 32-bit integer operations: the sum as a two's-complement integer of three words (h1, h0,
@@ -515,11 +518,12 @@ __device__ __forceinline__ void combine(const GemmParams& p, double& zr, double&
 // Epilogue of one 128 x 64 tile for G <= 8 groups (compile-time) over the tile's exactness
 // chunks: the exact sum of the group values v_g (|v| <= 2^24 per chunk) is H 2^(8 NL) + L with
 // H = the first NH = min(G, 4) groups and L = the rest (F64: the whole sum fits 64 bits, NL = 0 and
-// H takes every group, G <= 5), each accumulated over the chunks in 64 bits (|H|, |L| < 2^49 per
-// chunk).  A thread owns one row and 16 stacked columns (8 complex).  The groups are read two at a
-// time and released as soon as they are read, so the MMAs of the next chunk or tile start while
-// the rest is folded, rounded and written.  The outputs are rounded and combined in two halves of
-// 4 complex columns.
+// H takes every group, G <= 5), each accumulated over the chunks in 64 bits.  A thread owns one row and
+// 16 stacked columns (8 complex).  The groups are read two at a time.  Where their values are known to be
+// small (magic mask), a pair is released as soon as it is read; otherwise a part's groups are released
+// together, after the vote on their values and the second reading it may ask for.  Either way the MMAs of
+// the next chunk or tile start on them while the rest is folded, rounded and written.  The outputs are
+// rounded and combined in two halves of 4 complex columns.
 // Returns false if a wait gave up.
 // UPDATE: the mode combines with C (a separate instance: the values' registers would spill the others).
 template <int G, bool F64, bool KS, bool UPDATE>
